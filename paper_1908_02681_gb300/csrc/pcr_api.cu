@@ -27,11 +27,6 @@ struct pcr_framebuffer {
                              // per-pixel accept bounds (pcr::k_band_bounds)
   uint32_t* status;          // device status word
   pcr::Tuning tuning;        // launch tuning of the point passes
-  // device copy of the depth table of the view last rendered with the certified transform (loaded by the
-  // passes with coalesced reads), re-uploaded when the view changes
-  long long* d_table;
-  pcr::DevView table_view;
-  bool table_valid;
   // frames from host memory (pcr_render_frame_host): events, created by its first call (the copies go to the
   // device's upload queue, upload_stream)
   cudaEvent_t copy_events[9];  // [0]: start of the frame on the caller's stream; [1..8]: chunk k landed
@@ -166,28 +161,6 @@ pcr_status after_launch(const char* what, uint64_t launches = 1) {
   return e == cudaSuccess ? PCR_OK : cuda_fail(e, what);
 }
 
-// The device copy of the view's depth tables for the certified passes on fb (uploaded on `s` when the view
-// differs from the last one; one table, or one per PIECEWISE range), or null (double-float transform, FP64
-// kernels, or the upload failed: LINEAR and METRIC passes then read the table from their parameter block,
-// PIECEWISE views run on the FP64 kernels).
-const long long* fb_table(pcr_framebuffer* fb, const pcr::DevView& dv, int transform, cudaStream_t s) {
-  if (transform != PCR_TRANSFORM_EXACT) return nullptr;
-  const pcr::CertParams* P = nullptr;
-  const long long* tables = nullptr;
-  if (!pcr::cached_cert(dv, false, &P, &tables)) return nullptr;
-  if (!fb->table_valid || std::memcmp(&fb->table_view, &dv, sizeof(dv)) != 0) {
-    fb->table_valid = false;
-    if (cudaMemcpyAsync(fb->d_table, tables, pcr::table_blocks(*P) * sizeof(P->F), cudaMemcpyHostToDevice, s) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    fb->table_view = dv;
-    fb->table_valid = true;
-  }
-  return fb->d_table;
-}
-
 // A band mask request for pass 1: on, its eps, and where the launch's first tile sits in the mask (a pass 1
 // over a tile-aligned part of the frame's points).
 struct BandRequest {
@@ -239,11 +212,10 @@ pcr_status launch_raster(pcr_framebuffer* fb, const pcr_point* d_points, uint64_
     pcr::k_raster_fp64<<<grid_for(n, 256, fb->device, 8), 256, 0, s>>>(pts, n, dv, fb->keys);
     return after_launch("k_raster_fp64");
   }
-  const long long* table = fb_table(fb, dv, transform, s);
   const pcr::BandMask bm = pcr::band_mask(band.on ? fb->band_mask + 2 * band.tile_offset : nullptr, band.num,
                                           band.den, dv.nq);
   return pcr::launch_raster_certified(pts, n, dv, transform == PCR_TRANSFORM_DOUBLE_FLOAT, fb->keys, fb->status,
-                                      sm_count(fb->device), s, stats, fb->tuning, table, bm)
+                                      sm_count(fb->device), s, stats, fb->tuning, bm)
              ? after_launch("k_raster_certified")
              : fail(PCR_ERR_CUDA, "certified raster launch failed");
 }
@@ -291,14 +263,13 @@ pcr_status launch_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n,
     pcr::k_hq_fp64<<<grid_for(n, 256, fb->device, 8), 256, 0, s>>>(pts, n, dv, fb->keys, acc, eps_num, eps_den);
     return after_launch("k_hq_fp64");
   }
-  const long long* table = fb_table(fb, dv, transform, s);
   // pass 1's band mask, when it describes these points and view and an eps at least this one
   const bool band = fb->band_valid && transform == PCR_TRANSFORM_EXACT && fb->band_pts == d_points &&
                     fb->band_n == n && std::memcmp(&fb->band_view, &dv, sizeof(dv)) == 0 &&
                     (unsigned long long)eps_num * fb->band_den <= (unsigned long long)fb->band_num * eps_den;
   const int launched = pcr::launch_hq_certified(pts, n, dv, transform == PCR_TRANSFORM_DOUBLE_FLOAT, fb->keys, acc,
                                                 eps_num, eps_den, fb->status, sm_count(fb->device), s, fb->tuning,
-                                                table, band ? fb->band_mask : nullptr,
+                                                band ? fb->band_mask : nullptr,
                                                 fb->tuning.band_bounds ? bounds_buffer(fb, s) : nullptr);
   return after_launch("k_hq_certified", (uint64_t)launched);
 }
@@ -327,14 +298,12 @@ pcr_status pcr_create_framebuffer(int32_t width, int32_t height, uint32_t flags,
   e = cudaMalloc(&fb->keys, npx * sizeof(unsigned long long));
   if (e == cudaSuccess && (flags & PCR_FB_HQ)) e = cudaMalloc(&fb->accum, npx * sizeof(ulonglong2));
   if (e == cudaSuccess) e = cudaMalloc(&fb->status, 256);
-  if (e == cudaSuccess) e = cudaMalloc(&fb->d_table, pcr::kMaxRanges * sizeof(pcr::CertParams::F));
   if (e != cudaSuccess) {
     cudaGetLastError();
     cudaFree(fb->keys);
     cudaFree(fb->accum);
     cudaFree(fb->bounds);
     cudaFree(fb->status);
-    cudaFree(fb->d_table);
     delete fb;
     return e == cudaErrorMemoryAllocation ? fail(PCR_ERR_OOM, "cudaMalloc of %llu pixels failed", (unsigned long long)npx)
                                           : cuda_fail(e, "cudaMalloc");
@@ -365,7 +334,6 @@ pcr_status pcr_destroy_framebuffer(pcr_framebuffer* fb) {
   cudaFree(fb->accum);
   cudaFree(fb->bounds);
   cudaFree(fb->status);
-  cudaFree(fb->d_table);
   cudaFree(fb->band_mask);
   for (cudaEvent_t e : fb->copy_events)
     if (e) cudaEventDestroy(e);
@@ -521,24 +489,17 @@ pcr_status pcr_project_points(const pcr_point* d_points, uint64_t n, const pcr_v
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(d_key);
   const unsigned grid = grid_for(n, 256, device, 8);
   const pcr::CertParams* P = nullptr;
-  const long long* tables = nullptr;
   const bool approx = view->transform == PCR_TRANSFORM_DOUBLE_FLOAT;
-  if (view->transform == PCR_TRANSFORM_FP64 || !pcr::cached_cert(dv, approx, &P, &tables)) {
+  if (view->transform == PCR_TRANSFORM_FP64 || !pcr::cached_cert(dv, approx, &P)) {
     pcr::k_project_fp64<<<grid, 256, 0, s>>>(pts, n, dv, d_pixel, keys);
   } else if (P->n_pw > 0) {
-    // PIECEWISE: the ranges' tables in a stream-ordered temporary device copy
-    const size_t bytes = (size_t)P->n_pw * sizeof(P->F);
-    void* d_tab = nullptr;
-    cudaError_t e = cudaMallocAsync(&d_tab, bytes, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_tab, tables, bytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) {
-      auto kernel = P->n_pw > 2 ? pcr::k_project_cert<false, 2> : pcr::k_project_cert<false, 1>;
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      if (e == cudaSuccess) kernel<<<grid, 256, bytes, s>>>(pts, n, *P, d_pixel, keys, (const long long*)d_tab);
-      if (e == cudaSuccess) e = cudaGetLastError();
-    }
-    if (d_tab) cudaFreeAsync(d_tab, s);
+    const size_t bytes = (size_t)P->n_pw * pcr::kTableBytes;  // PIECEWISE: the ranges' tables
+    auto kernel = P->n_pw > 2 ? pcr::k_project_cert<false, 2> : pcr::k_project_cert<false, 1>;
+    // opt in to the largest size, so that a concurrent call with fewer ranges does not lower the limit
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(pcr::kMaxRanges * pcr::kTableBytes));
     if (e != cudaSuccess) return cuda_fail(e, "piecewise projection");
+    kernel<<<grid, 256, bytes, s>>>(pts, n, *P, d_pixel, keys);
   } else if (approx)
     pcr::k_project_cert<true><<<grid, 256, 0, s>>>(pts, n, *P, d_pixel, keys);
   else

@@ -12,7 +12,7 @@
 //     never skipped.
 //   * one persistent launch per pass for all views: work items are (range of consecutive chunks, view),
 //     taken range by range from a counter, so a range is read from HBM once for all views; a block
-//     reloads a view's depth table when its view changes. The range size, points per thread, grid size and
+//     rebuilds its depth table when its view changes. The range size, points per thread, grid size and
 //     same-pixel merging are launch tuning (BatchTuning), picked by an autotuner (pcr_batch_autotune).
 //   * one resolve launch for all views.
 #pragma once
@@ -201,11 +201,9 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
     const uint32_t nvis = s_nvis;
     if (nvis == 0u) continue;  // nothing of this range is visible in this view (the same in every thread)
     if (v != cur_view) {
-      const long long* src = &params[v].F[0][0];
-      for (int i = threadIdx.x; i < 3 * kTableEntries; i += blockDim.x) sF[i] = src[i];
+      build_tables(params[v].col, 1, sF);
       cur_view = v;
     }
-    __syncthreads();
     const CertParams& Pg = params[v];
     const HotParams H = hot_params(Pg);
     const BatchSlot& S = slots[v];

@@ -8,8 +8,8 @@
 //   * depth code: t = S * (w - near) (LINEAR, S = s) or S * w (METRIC, S = metric_scale) is linear in the
 //     point, t = sum_j A_j X_j + B with A_j = S * M[3][j]. Each float coordinate X_j = m_j * 2^(e_j - 150)
 //     (24-bit integer mantissa m_j, biased exponent e_j), so A_j X_j = m_j * (A_j * 2^(e_j - 150)). A
-//     per-view table holds round(A_j * 2^(e - 150) * 2^40) for every sign and exponent (built exactly on
-//     the host with 128-bit integers); the point's t * 2^40 is the 96-bit integer sum of three 24x64-bit
+//     per-view table holds round(A_j * 2^(e - 150) * 2^40) for every sign and exponent (built exactly by each
+//     block in shared memory, see depth_entry); the point's t * 2^40 is the 96-bit integer sum of three 24x64-bit
 //     products and B * 2^40, within 2^-15 of the exact real t. The FP64 definition's own rounding moves t
 //     by at most u64 * (5.2 * T_t + 3.1 * S * near), T_t = sum |A_j X_j| + |B|; when the interval of
 //     both errors around the integer sum holds no integer, floor(t_FP64) is known exactly.
@@ -45,11 +45,44 @@ namespace pcr {
 constexpr int kTableExp = 256;                 // biased float exponents
 constexpr int kTableEntries = 2 * kTableExp;   // x sign
 constexpr int kFixedFracBits = 40;             // t is held in units of 2^-40
+constexpr size_t kTableBytes = 3 * kTableEntries * sizeof(long long);  // one depth table (three coordinates)
 
-// Per-view constants of the certified evaluation. Passed by value as a __grid_constant__ kernel
-// parameter (about 12.8 KB), so concurrent launches with different views share nothing.
+// One coordinate's column of a depth table, as the exact product of the two doubles it comes from: S * M[3][j] =
+// (neg ? -1 : 1) * (hi 2^64 + lo) * 2^k, an integer of `bits` bits (0: the column is zero), with the exponents
+// folded into sh: entry e is round((hi 2^64 + lo) * 2^(sh + e)).
+struct DepthColumn {
+  unsigned long long lo, hi;
+  int32_t sh, bits;
+  int32_t neg, pad;
+};
+
+// |F[j][e]| of a column: the product shifted by sh + e (subnormals, e = 0, share exponent 1's scale), rounded half
+// up. False when the entry would reach 2^62 (or e is the exponent of infinities): it is then not usable and 0.
+__host__ __device__ __forceinline__ bool depth_entry(const DepthColumn& c, int e, unsigned long long* mag) {
+  const int s = c.sh + (e == 0 ? 1 : e);
+  *mag = 0ull;
+  if (e >= kTableExp - 1) return false;
+  if (c.bits == 0) return true;
+  if (c.bits + s > 62) return false;
+  if (s >= 0) {  // at most 62 bits in all: hi is 0
+    *mag = c.lo << s;
+    return true;
+  }
+  const int n = -s - 1;  // half up: ((product >> n) + 1) >> 1, product >> n below 2^63
+  const unsigned long long q = n >= 128 ? 0ull : n >= 64 ? c.hi >> (n - 64) : n == 0 ? c.lo : (c.lo >> n) | (c.hi << (64 - n));
+  const unsigned long long m = (q + 1ull) >> 1;
+  if (m >> 62) return false;
+  *mag = m;
+  return true;
+}
+
+// Per-view constants of the certified evaluation. Passed by value as a __grid_constant__ kernel parameter (about
+// 1.9 KB), so concurrent launches with different views share nothing. The depth tables (12 KB a view or PIECEWISE
+// range) are not in it: every block builds them from the columns below (build_tables). They used to be built on the
+// host (14 us a view), copied to the device and read by each block: a frame with a new camera over 40,000 points took
+// 37 us that way and takes 26 us now, 1M points at 640x480 36 us and now 23 us.
 struct CertParams {
-  // hot scalars first: the per-point loops read them as instruction operands; the table comes last
+  // hot scalars first: the per-point loops read them as instruction operands; the columns come last
   float H[3][4], L[3][4];             // float splits of the rows clip x, clip y, w (H: nearest float, L: rest)
   // tier 1 (classify_fast); s = |x| + |y| + |z| of the point, evaluated in float
   float Wr[4];                        // w row, nearest floats of M[3][c]
@@ -74,7 +107,7 @@ struct CertParams {
   int32_t approximate;
   int32_t linear;
   // PIECEWISE depth: the n_pw ranges that meet [near, far) (0: LINEAR or METRIC). Range r has its own depth
-  // table (block r of the device table, 3 * kTableEntries entries each), window, code margin and first code.
+  // table (columns col[r], 3 * kTableEntries entries), window, code margin and first code.
   int32_t n_pw;
   float pw_wc[kMaxRanges], pw_whk[kMaxRanges], pw_kd[kMaxRanges], pw_hd0[kMaxRanges];
   float pw_start[kMaxRanges];         // ascending split points: range r is the only one whose window may hold
@@ -82,7 +115,7 @@ struct CertParams {
   unsigned long long pw_BL[kMaxRanges];  // (B_r + base_r 2^40) = BH 2^32 + BL: the first code folded in
   long long pw_BH[kMaxRanges];
   DevView v;                          // the FP64 definition (for the arbiter)
-  long long F[3][kTableEntries];      // t-row fixed-point coefficients, index (sign << 8) | exponent
+  DepthColumn col[kMaxRanges][3];     // the tables' columns, row r for PIECEWISE range r (row 0: LINEAR, METRIC)
 };
 
 // The first-tier constants of one view (a subset of CertParams with the same field names).
@@ -274,28 +307,31 @@ inline bool tier1_constants(const DevView& v, double S, CertParams* P) {
   return true;
 }
 
-// The fixed-point depth table of t = S (w - off): F[j][(sign << 8) | e] = round(S M[3][j] 2^(e - 150) 2^40) for
-// every sign and biased exponent of coordinate j (0 past the largest usable exponent, which goes to e_max[j]),
-// and b = S (M[3][3] - off) 2^40 rounded. False when the scale puts the values out of the representable range.
-inline bool build_table(double S, const double* m3, double off, long long (*F)[kTableEntries], int32_t* e_max,
-                        __int128* b_out) {
+// The columns of the fixed-point depth table of t = S (w - off): F[j][(sign << 8) | e] = round(S M[3][j]
+// 2^(e - 150) 2^40) for every sign and biased exponent of coordinate j (0 past the largest usable exponent, which
+// goes to e_max[j]), and b = S (M[3][3] - off) 2^40 rounded. False when the scale puts the values out of the
+// representable range.
+inline bool table_columns(double S, const double* m3, double off, DepthColumn* col, int32_t* e_max, __int128* b_out) {
   for (int j = 0; j < 3; ++j) {
     const double a = S * m3[j];
     if (!(std::fabs(a) < 0x1p80)) return false;  // keeps the subnormal shortcut's error below 2^-46
-    e_max[j] = 254;
-    for (int e = 0; e < kTableExp; ++e) {
-      const int ee = e == 0 ? 1 : e;  // subnormals share exponent 1's scale (see the device loop)
-      __int128 f;
-      const bool ok = e < 255 && fixed_mul(S, m3[j], ee - 150 + kFixedFracBits, &f) &&
-                      f < ((__int128)1 << 62) && f > -((__int128)1 << 62);
-      if (!ok) {
-        if (e_max[j] >= e) e_max[j] = e - 1;
-        f = 0;
-      }
-      F[j][e] = (long long)f;
-      F[j][kTableExp + e] = -(long long)f;
-    }
-    if (e_max[j] < 127) return false;  // coordinates of magnitude 1 would not be usable
+    DepthColumn& c = col[j];
+    std::memset(&c, 0, sizeof(c));
+    int es, em;
+    const double fs = std::frexp(S, &es), fm = std::frexp(m3[j], &em);
+    const long long ms = (long long)std::ldexp(fs, 53), mm = (long long)std::ldexp(fm, 53);  // exact
+    const unsigned __int128 p = (unsigned __int128)(ms < 0 ? -ms : ms) * (unsigned __int128)(mm < 0 ? -mm : mm);
+    c.lo = (unsigned long long)p;
+    c.hi = (unsigned long long)(p >> 64);
+    c.neg = (ms < 0) != (mm < 0) ? 1 : 0;
+    c.bits = c.hi ? 128 - __builtin_clzll(c.hi) : c.lo ? 64 - __builtin_clzll(c.lo) : 0;
+    c.sh = es - 53 + em - 53 - 150 + kFixedFracBits;
+    // entries grow with e: the last usable one is at most one below the first exponent that fills 62 bits
+    unsigned long long mag;
+    int e = c.bits == 0 || 62 - c.bits - c.sh > 254 ? 254 : 62 - c.bits - c.sh;
+    while (e >= 127 && !depth_entry(c, e, &mag)) --e;
+    if (e < 127) return false;  // coordinates of magnitude 1 would not be usable
+    e_max[j] = e;
   }
   __int128 b, bn = 0;
   if (!fixed_mul(S, m3[3], kFixedFracBits, &b)) return false;
@@ -343,16 +379,14 @@ inline bool piecewise_range(double res, double lo, double lo_e, double hi_e, dou
 }
 
 // Fills P for the view; false when the view is outside the certified evaluation's preconditions (the
-// caller then uses the FP64 kernels, which accept every valid view). tables (may be null): receives the
-// depth tables, block r for PIECEWISE range r (block 0 is P->F for LINEAR and METRIC).
-inline bool prepare_cert(const DevView& v, bool approximate, CertParams* P,
-                         long long (*tables)[3][kTableEntries] = nullptr) {
+// caller then uses the FP64 kernels, which accept every valid view).
+inline bool prepare_cert(const DevView& v, bool approximate, CertParams* P) {
   std::memset(P, 0, sizeof(*P));
   P->v = v;
   P->approximate = approximate ? 1 : 0;
   const bool pw = v.depth_mode == 2;
   if (v.depth_mode != 0 && v.depth_mode != 1 && !pw) return false;
-  if (pw && (approximate || !tables)) return false;  // piecewise: the exact transform with device tables only
+  if (pw && approximate) return false;  // piecewise: the exact transform only
   P->linear = v.depth_mode != 1;
   if (!(v.near_ >= 0x1p-60) || !(v.far_ < 0x1p100)) return false;
   for (int r = 0; r < 3; ++r)
@@ -376,7 +410,7 @@ inline bool prepare_cert(const DevView& v, bool approximate, CertParams* P,
       }
       int32_t em[3];
       __int128 b;
-      if (!build_table(res, m3, v.lo[k], tables[n], em, &b)) return false;
+      if (!table_columns(res, m3, v.lo[k], P->col[n], em, &b)) return false;
       for (int j = 0; j < 3; ++j) emin[j] = em[j] < emin[j] ? em[j] : emin[j];
       b += (__int128)(unsigned long long)v.base[k] << kFixedFracBits;  // codes of range k start at base_k
       P->pw_BL[n] = (unsigned long long)(uint32_t)(unsigned __int128)b;
@@ -385,11 +419,10 @@ inline bool prepare_cert(const DevView& v, bool approximate, CertParams* P,
       ++n;
     }
     if (n == 0) return false;  // nothing of [near, far) has a code: every point is culled (FP64 kernels)
-    // one range: NaN, so that no w (+inf included) selects the second arm, whose table the kernels do not hold
+    // one range: NaN, so that no w (+inf included) selects the second arm, whose table the kernels do not build
     if (n == 1) P->pw_start[1] = std::nanf("");
     P->n_pw = n;
     P->xyz_max = xyz_limit(emin);
-    std::memcpy(P->F, tables[0], sizeof(P->F));
     P->BL = P->pw_BL[0];
     P->BH = P->pw_BH[0];
     return true;
@@ -402,7 +435,7 @@ inline bool prepare_cert(const DevView& v, bool approximate, CertParams* P,
   // t = sum_j A_j X_j + B, A_j = S * M[3][j], B = S * (M[3][3] - near) (LINEAR) or S * M[3][3] (METRIC)
   for (int j = 0; j < 3; ++j) P->Af[j] = (float)(S * m3[j]);
   __int128 b;
-  if (!build_table(S, m3, P->linear ? v.near_ : 0.0, P->F, P->e_max, &b)) return false;
+  if (!table_columns(S, m3, P->linear ? v.near_ : 0.0, P->col[0], P->e_max, &b)) return false;
   const unsigned __int128 bu = (unsigned __int128)b;
   P->B0 = (uint32_t)bu;
   P->B1 = (uint32_t)(bu >> 32);
@@ -428,7 +461,6 @@ inline bool prepare_cert(const DevView& v, bool approximate, CertParams* P,
   P->qn_cull = (long long)std::floor(Tn) - 1;
   P->qf_safe = (long long)std::floor(Tf) - 1;
   P->qf_cull = (long long)std::floor(Tf) + 1;
-  if (tables) std::memcpy(tables[0], P->F, sizeof(P->F));
   return true;
 }
 
@@ -528,8 +560,7 @@ __device__ __forceinline__ uint32_t depth_decision(const CertParams& P, long lon
   return exact ? kExact : kAmbiguous;
 }
 
-// Tier 2: certified double-float clip values (see the file header). F points at the block's
-// shared-memory copy of P.F.
+// Tier 2: certified double-float clip values (see the file header). F points at the block's depth table.
 __device__ __forceinline__ CertFrag classify_cert(const CertParams& P, const long long* __restrict__ F, uint4 p) {
   CertFrag out{kCulled, 0u, 0};
   if (P.n_pw) {  // PIECEWISE: a point tier 1 could not decide goes to the FP64 definition
@@ -775,20 +806,24 @@ __device__ __forceinline__ CertFrag classify_df(const CertParams& P, uint4 p) {
   return out;
 }
 
-__device__ __forceinline__ void load_table(const CertParams& P, long long* sF) {
-  const long long* src = &P.F[0][0];
-  for (int i = threadIdx.x; i < 3 * kTableEntries; i += blockDim.x) sF[i] = src[i];
-  __syncthreads();
-}
-
-// The same table from a device-memory copy (coalesced loads; from the kernel parameter block, every lane
-// reading its own address, the copy took ~14 us per launch). table == null: from the parameter block.
-__device__ __forceinline__ void load_table(const CertParams& P, const long long* __restrict__ table, long long* sF) {
-  if (table == nullptr) {
-    load_table(P, sF);
-    return;
+// Builds `blocks` depth tables (PIECEWISE: one per range) from their columns in the block's shared memory: each
+// thread shifts and rounds the columns' products for its exponents and writes both signs. A 256-thread block
+// computes 3 entries a thread a table, about 40 integer instructions each, in place of 6 dependent loads from L2.
+__device__ __forceinline__ void build_tables(const DepthColumn (*col)[3], int blocks, long long* sF) {
+  for (int r = 0; r < blocks; ++r) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const DepthColumn& c = col[r][j];
+      long long* const row = sF + (3 * r + j) * kTableEntries;
+      for (int e = threadIdx.x; e < kTableExp; e += blockDim.x) {
+        unsigned long long mag;
+        depth_entry(c, e, &mag);
+        const long long f = c.neg ? -(long long)mag : (long long)mag;
+        row[e] = f;
+        row[kTableExp + e] = -f;
+      }
+    }
   }
-  for (int i = threadIdx.x; i < 3 * kTableEntries; i += blockDim.x) sF[i] = table[i];
   __syncthreads();
 }
 
@@ -1044,7 +1079,7 @@ __device__ __forceinline__ void defer_points(bool defer, const uint4& p, uint4* 
 // Pass 1 (Section 2.1) with the certified transform. Tier 1 handles nearly every point; the others are
 // queued per warp in shared memory and handled 32 at a time by tier 2 and the FP64 arbiter. The points
 // arrive through stream_tiles (direct loads or bulk-copy rings). kPw > 0: PIECEWISE depth (see classify_fast),
-// the ranges' tables in dynamic shared memory (P.n_pw blocks of 3 * kTableEntries entries, from the device table).
+// the ranges' tables in dynamic shared memory (P.n_pw blocks of 3 * kTableEntries entries).
 // kBand: also writes the band mask for pass 2 (band.mask: two words per tile of 64 points, bit lane of word
 // 2 tile + k for point 64 tile + 32 k + lane): the bit is clear when the point is culled, or when its key is
 // certainly outside the final band of eps = eps_num / eps_den = E + f (E integer, 0 <= f < 1). The test takes
@@ -1089,7 +1124,7 @@ template <bool kApprox, bool kMerge, bool kStats, bool kRing, int kPw, bool kBan
 __global__ void __launch_bounds__(kCertThreads, kApprox ? PCR_CERT_APPROX_MIN_BLOCKS : PCR_CERT_MIN_BLOCKS) k_raster_cert(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P,
     unsigned long long* __restrict__ keys, unsigned long long* __restrict__ stats, uint32_t* __restrict__ status,
-    const long long* __restrict__ table, BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
+    BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
   __shared__ long long sF_static[kPw ? 1 : 3 * kTableEntries];
   extern __shared__ __align__(16) long long sF_dynamic[];
   __shared__ uint4 queue[kCertWarps][kQueue];
@@ -1099,12 +1134,7 @@ __global__ void __launch_bounds__(kCertThreads, kApprox ? PCR_CERT_APPROX_MIN_BL
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   if (kRing && lane == 0) ring_init(bars[warp]);
   __syncwarp();
-  if constexpr (kPw) {
-    for (int i = threadIdx.x; i < P.n_pw * 3 * kTableEntries; i += blockDim.x) sF[i] = table[i];
-    __syncthreads();
-  } else if (!kApprox) {
-    load_table(P, table, sF);
-  }
+  if (!kApprox) build_tables(P.col, kPw ? P.n_pw : 1, sF);
   uint4* q = queue[warp];
   uint32_t qn = 0;
   unsigned c_exact = 0, c_amb = 0, c_fp64 = 0, c_defer = 0;
@@ -1322,8 +1352,7 @@ template <bool kApprox, bool kMerge, bool kRing, bool kBand = false>
 __global__ void __launch_bounds__(kCertThreads, PCR_HQ_MIN_BLOCKS) k_hq_cert(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P,
     const unsigned long long* __restrict__ keys, unsigned long long* __restrict__ accum, uint32_t eps_num,
-    uint32_t eps_den, uint32_t* __restrict__ status, const long long* __restrict__ table,
-    const uint32_t* __restrict__ band_mask = nullptr, const ulonglong2* __restrict__ bounds = nullptr) {
+    uint32_t eps_den, uint32_t* __restrict__ status, const uint32_t* __restrict__ band_mask = nullptr, const ulonglong2* __restrict__ bounds = nullptr) {
   __shared__ long long sF[3 * kTableEntries];
   __shared__ uint4 queue[kCertWarps][kQueue];
   __shared__ uint4 cand_queue[kBand ? kCertWarps : 1][kQueue];
@@ -1332,7 +1361,7 @@ __global__ void __launch_bounds__(kCertThreads, PCR_HQ_MIN_BLOCKS) k_hq_cert(
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   if (kRing && lane == 0) ring_init(bars[warp]);
   __syncwarp();
-  if (!kApprox) load_table(P, table, sF);
+  if (!kApprox) build_tables(P.col, 1, sF);
   uint4* q = queue[warp];
   uint32_t qn = 0;
   // The additions of accepted fragments: warp-level same-pixel merging (kMerge), else lane pairs.
@@ -1474,93 +1503,77 @@ inline unsigned persistent_grid(int resident, uint64_t n, int sms, int per_sm) {
   return cert_grid(n, sms, per_sm < resident ? per_sm : resident);
 }
 
-// table: device copy of P.F (or null: the kernels read it from the parameter block); for PIECEWISE views
-// (P.n_pw > 0) the device copy of all the ranges' tables, required.
 template <bool kApprox, bool kMerge, bool kStats, bool kRing, int kPw, bool kBand = false>
 inline void raster_launch5(const uint4* pts, uint64_t n, const CertParams& P, unsigned long long* keys,
                            unsigned long long* stats, uint32_t* status, int sms, int per_sm, cudaStream_t s,
-                           const long long* table, BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
+                           BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
   auto kernel = k_raster_cert<kApprox, kMerge, kStats, kRing, kPw, kBand>;
   if constexpr (kPw) {
     // the ranges' tables in dynamic shared memory: up to kMaxRanges * 12 KB (opt in above 48 KB once)
     static const bool opted = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)(kMaxRanges * sizeof(P.F))) == cudaSuccess;
+                                                   (int)(kMaxRanges * kTableBytes)) == cudaSuccess;
     (void)opted;
-    const size_t dyn = (size_t)P.n_pw * sizeof(P.F);
+    const size_t dyn = (size_t)P.n_pw * kTableBytes;
     int resident = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kCertThreads, dyn) != cudaSuccess ||
         resident < 1) {
       cudaGetLastError();
       resident = 1;
     }
-    kernel<<<persistent_grid(resident, n, sms, per_sm), kCertThreads, dyn, s>>>(pts, n, P, keys, stats, status, table,
-                                                                               band);
+    kernel<<<persistent_grid(resident, n, sms, per_sm), kCertThreads, dyn, s>>>(pts, n, P, keys, stats, status, band);
   } else {
     static const int resident = resident_blocks(kernel);  // per instantiation
-    kernel<<<persistent_grid(resident, n, sms, per_sm), kCertThreads, 0, s>>>(pts, n, P, keys, stats, status, table,
-                                                                             band);
+    kernel<<<persistent_grid(resident, n, sms, per_sm), kCertThreads, 0, s>>>(pts, n, P, keys, stats, status, band);
   }
 }
 
 template <bool kApprox, bool kMerge, bool kStats, bool kRing>
 inline void raster_launch4(const uint4* pts, uint64_t n, const CertParams& P, unsigned long long* keys,
                            unsigned long long* stats, uint32_t* status, int sms, int per_sm, cudaStream_t s,
-                           const long long* table, BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
+                           BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
   if constexpr (!kApprox && !kStats) {
     if (band.mask && P.n_pw == 0) {  // also write the band mask for pass 2
-      raster_launch5<false, kMerge, false, kRing, 0, true>(pts, n, P, keys, nullptr, status, sms, per_sm, s, table,
-                                                           band);
+      raster_launch5<false, kMerge, false, kRing, 0, true>(pts, n, P, keys, nullptr, status, sms, per_sm, s, band);
       return;
     }
   }
   if (!kApprox && P.n_pw > 2)
-    raster_launch5<false, kMerge, kStats, kRing, 2>(pts, n, P, keys, stats, status, sms, per_sm, s, table);
+    raster_launch5<false, kMerge, kStats, kRing, 2>(pts, n, P, keys, stats, status, sms, per_sm, s);
   else if (!kApprox && P.n_pw > 0)
-    raster_launch5<false, kMerge, kStats, kRing, 1>(pts, n, P, keys, stats, status, sms, per_sm, s, table);
+    raster_launch5<false, kMerge, kStats, kRing, 1>(pts, n, P, keys, stats, status, sms, per_sm, s);
   else
-    raster_launch5<kApprox, kMerge, kStats, kRing, 0>(pts, n, P, keys, stats, status, sms, per_sm, s, table);
+    raster_launch5<kApprox, kMerge, kStats, kRing, 0>(pts, n, P, keys, stats, status, sms, per_sm, s);
 }
 
 // Pass 1 with the tuning's staging; the tier counters (stats) only with the exact transform, no merging.
 template <bool kApprox, bool kMerge>
 inline void raster_launch(const uint4* pts, uint64_t n, const CertParams& P, unsigned long long* keys,
                           unsigned long long* stats, uint32_t* status, int sms, int per_sm, cudaStream_t s,
-                          const long long* table = nullptr, int staging = 0,
+                          int staging = 0,
                           BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
   if (stats && !kApprox && !kMerge)
-    staging ? raster_launch4<false, false, true, true>(pts, n, P, keys, stats, status, sms, per_sm, s, table)
-            : raster_launch4<false, false, true, false>(pts, n, P, keys, stats, status, sms, per_sm, s, table);
+    staging ? raster_launch4<false, false, true, true>(pts, n, P, keys, stats, status, sms, per_sm, s)
+            : raster_launch4<false, false, true, false>(pts, n, P, keys, stats, status, sms, per_sm, s);
   else
-    staging ? raster_launch4<kApprox, kMerge, false, true>(pts, n, P, keys, nullptr, status, sms, per_sm, s, table,
-                                                           band)
-            : raster_launch4<kApprox, kMerge, false, false>(pts, n, P, keys, nullptr, status, sms, per_sm, s, table,
-                                                            band);
+    staging ? raster_launch4<kApprox, kMerge, false, true>(pts, n, P, keys, nullptr, status, sms, per_sm, s, band)
+            : raster_launch4<kApprox, kMerge, false, false>(pts, n, P, keys, nullptr, status, sms, per_sm, s, band);
 }
 
 // The certified constants of a view, prepared on this thread and kept for the next call with the same view
-// and mode (prepare_cert builds a 12 KB exact table: ~14 us of host time per call). Returns false when the
-// view is outside the single-precision preconditions.
-// tables (optional): the view's depth tables, block r for PIECEWISE range r (P->n_pw blocks; one for LINEAR
-// and METRIC), to be copied to the device.
-inline bool cached_cert(const DevView& v, bool approximate, const CertParams** out,
-                        const long long** tables = nullptr) {
+// and mode. Returns false when the view is outside the single-precision preconditions.
+inline bool cached_cert(const DevView& v, bool approximate, const CertParams** out) {
   static thread_local CertParams P;
-  static thread_local long long T[kMaxRanges][3][kTableEntries];
   static thread_local DevView last_v;
   static thread_local int last = -1;  // -1: nothing cached; else approximate (0/1) of the cached view
   static thread_local bool last_ok = false;
   if (last != (approximate ? 1 : 0) || std::memcmp(&last_v, &v, sizeof(DevView)) != 0) {
-    last_ok = host::prepare_cert(v, approximate, &P, T);
+    last_ok = host::prepare_cert(v, approximate, &P);
     std::memcpy(&last_v, &v, sizeof(DevView));
     last = approximate ? 1 : 0;
   }
   *out = &P;
-  if (tables) *tables = &T[0][0][0];
   return last_ok;
 }
-
-// Blocks of the depth tables of prepared constants (the device copy's size in tables of 3 * kTableEntries).
-inline int table_blocks(const CertParams& P) { return P.n_pw > 0 ? P.n_pw : 1; }
 
 // Pass 1 for a view with n >= 1 points. status: the framebuffer's status word (timeout bit).
 // band (mask non-null): also write the band mask for pass 2 (used only with the exact transform on LINEAR or
@@ -1568,33 +1581,31 @@ inline int table_blocks(const CertParams& P) { return P.n_pw > 0 ? P.n_pw : 1; }
 inline bool launch_raster_certified(const uint4* pts, uint64_t n, const DevView& v, bool approximate,
                                     unsigned long long* keys, uint32_t* status, int sms, cudaStream_t s,
                                     unsigned long long* stats = nullptr, const Tuning& t = Tuning(),
-                                    const long long* table = nullptr, BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
+                                    BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
   const CertParams* Pp = nullptr;
   const unsigned grid = cert_grid(n, sms, t.blocks_per_sm);
-  // PIECEWISE views need the device copy of their tables
-  if (!cached_cert(v, approximate, &Pp) || (Pp->n_pw > 0 && table == nullptr)) {
+  if (!cached_cert(v, approximate, &Pp)) {
     k_raster_fp64<<<grid, 256, 0, s>>>(pts, n, v, keys);
     return true;
   }
   const int b = t.blocks_per_sm, g = t.staging;
   if (approximate)
-    t.merge ? raster_launch<true, true>(pts, n, *Pp, keys, stats, status, sms, b, s, table, g)
-            : raster_launch<true, false>(pts, n, *Pp, keys, stats, status, sms, b, s, table, g);
+    t.merge ? raster_launch<true, true>(pts, n, *Pp, keys, stats, status, sms, b, s, g)
+            : raster_launch<true, false>(pts, n, *Pp, keys, stats, status, sms, b, s, g);
   else
-    t.merge ? raster_launch<false, true>(pts, n, *Pp, keys, stats, status, sms, b, s, table, g, band)
-            : raster_launch<false, false>(pts, n, *Pp, keys, stats, status, sms, b, s, table, g, band);
+    t.merge ? raster_launch<false, true>(pts, n, *Pp, keys, stats, status, sms, b, s, g, band)
+            : raster_launch<false, false>(pts, n, *Pp, keys, stats, status, sms, b, s, g, band);
   return true;
 }
 
 template <bool kApprox, bool kMerge, bool kRing, bool kBand = false>
 inline void hq_launch4(const uint4* pts, uint64_t n, const CertParams& P, const unsigned long long* keys,
                        unsigned long long* accum, uint32_t eps_num, uint32_t eps_den, uint32_t* status, int sms,
-                       int per_sm, cudaStream_t s, const long long* table, const uint32_t* band_mask,
-                       const ulonglong2* bounds) {
+                       int per_sm, cudaStream_t s, const uint32_t* band_mask, const ulonglong2* bounds) {
   static const int resident = resident_blocks(k_hq_cert<kApprox, kMerge, kRing, kBand>);  // one per instantiation
   const unsigned grid = persistent_grid(resident, n, sms, per_sm);
   k_hq_cert<kApprox, kMerge, kRing, kBand><<<grid, kCertThreads, 0, s>>>(pts, n, P, keys, accum, eps_num, eps_den,
-                                                                         status, table, band_mask, bounds);
+                                                                         status, band_mask, bounds);
 }
 
 // band_mask (exact transform only): pass 1's band mask of the same points and view, or null. bounds (exact
@@ -1602,22 +1613,20 @@ inline void hq_launch4(const uint4* pts, uint64_t n, const CertParams& P, const 
 template <bool kApprox, bool kMerge>
 inline void hq_launch(const uint4* pts, uint64_t n, const CertParams& P, const unsigned long long* keys,
                       unsigned long long* accum, uint32_t eps_num, uint32_t eps_den, uint32_t* status, int sms,
-                      int per_sm, cudaStream_t s, const long long* table = nullptr, int staging = 0,
+                      int per_sm, cudaStream_t s, int staging = 0,
                       const uint32_t* band_mask = nullptr, const ulonglong2* bounds = nullptr) {
   if constexpr (!kApprox) {
     if (band_mask) {
-      staging ? hq_launch4<false, kMerge, true, true>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s,
-                                                      table, band_mask, bounds)
-              : hq_launch4<false, kMerge, false, true>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm,
-                                                       s, table, band_mask, bounds);
+      staging ? hq_launch4<false, kMerge, true, true>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s, band_mask, bounds)
+              : hq_launch4<false, kMerge, false, true>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s, band_mask, bounds);
       return;
     }
   } else {
     bounds = nullptr;
   }
-  staging ? hq_launch4<kApprox, kMerge, true>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s, table,
+  staging ? hq_launch4<kApprox, kMerge, true>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s,
                                               nullptr, bounds)
-          : hq_launch4<kApprox, kMerge, false>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s, table,
+          : hq_launch4<kApprox, kMerge, false>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s,
                                                nullptr, bounds);
 }
 
@@ -1628,8 +1637,7 @@ inline void hq_launch(const uint4* pts, uint64_t n, const CertParams& P, const u
 inline int launch_hq_certified(const uint4* pts, uint64_t n, const DevView& v, bool approximate,
                                const unsigned long long* keys, unsigned long long* accum, uint32_t eps_num,
                                uint32_t eps_den, uint32_t* status, int sms, cudaStream_t s,
-                               const Tuning& t = Tuning(), const long long* table = nullptr,
-                               const uint32_t* band_mask = nullptr, ulonglong2* bounds_buf = nullptr) {
+                               const Tuning& t = Tuning(), const uint32_t* band_mask = nullptr, ulonglong2* bounds_buf = nullptr) {
   const CertParams* Pp = nullptr;
   const unsigned grid = cert_grid(n, sms, t.blocks_per_sm);
   if (!cached_cert(v, approximate, &Pp) || Pp->n_pw > 0) {  // (HQ takes LINEAR or METRIC views only)
@@ -1638,8 +1646,8 @@ inline int launch_hq_certified(const uint4* pts, uint64_t n, const DevView& v, b
   }
   const int b = t.blocks_per_sm, g = t.staging;
   if (approximate) {
-    t.merge ? hq_launch<true, true>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, table, g)
-            : hq_launch<true, false>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, table, g);
+    t.merge ? hq_launch<true, true>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g)
+            : hq_launch<true, false>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g);
     return 1;
   }
   const ulonglong2* bounds = nullptr;
@@ -1649,9 +1657,9 @@ inline int launch_hq_certified(const uint4* pts, uint64_t n, const DevView& v, b
     k_band_bounds<<<bgrid, 256, 0, s>>>(keys, npx, v.nq, eps_num, div_magic(eps_den), bounds_buf);
     bounds = bounds_buf;
   }
-  t.merge ? hq_launch<false, true>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, table, g,
+  t.merge ? hq_launch<false, true>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g,
                                    band_mask, bounds)
-          : hq_launch<false, false>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, table, g,
+          : hq_launch<false, false>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g,
                                     band_mask, bounds);
   return bounds ? 2 : 1;
 }
