@@ -98,10 +98,11 @@ typedef struct {
 typedef struct {
   int32_t merge_same_pixel; /* 1: the fragments of one warp that land on the same pixel are merged with warp
                                reductions, then one atomic per pixel; 0 (default): pass 1 issues one atomic
-                               per fragment whose key is below the key the pixel holds, and pass 2 merges the
-                               additions of two adjacent lanes (consecutive points) that land on one pixel */
+                               per fragment that may be below the key the pixel holds, and pass 2 merges the
+                               additions of neighbouring accepted fragments that land on one pixel */
   int32_t blocks_per_sm;    /* 256-thread blocks per SM for the point passes, 1..32 (default 8; capped at the
-                               blocks that can be resident, 4 for pass 1 and 5 for pass 2) */
+                               threads that can be resident: 1024 per SM for the passes of default tuning, which
+                               run them as one block, else 4 blocks for pass 1 and 5 for pass 2) */
   int32_t staging;          /* how each warp brings its tiles of 64 points in: 0 (default) its own 16-byte
                                loads, one tile ahead; 1 bulk copies (cp.async.bulk) into a two-stage
                                shared-memory ring whose waits are bounded (a wait that gives up sets the

@@ -16,6 +16,7 @@
 #include "pcr_certified.cuh"
 #include "pcr_kernels.cuh"
 #include "pcr_project.cuh"
+#include "pcr_screen.cuh"
 
 struct pcr_framebuffer {
   int32_t width, height;
@@ -256,7 +257,7 @@ ulonglong2* bounds_buffer(pcr_framebuffer* fb, cudaStream_t s) {
 }
 
 pcr_status launch_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr::DevView& dv,
-                     int transform, uint32_t eps_num, uint32_t eps_den, cudaStream_t s) {
+                     int transform, uint32_t eps_num, uint32_t eps_den, cudaStream_t s, bool own_pass1) {
   const uint4* pts = reinterpret_cast<const uint4*>(d_points);
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(fb->accum);
   if (transform == PCR_TRANSFORM_FP64) {
@@ -270,7 +271,7 @@ pcr_status launch_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n,
   const int launched = pcr::launch_hq_certified(pts, n, dv, transform == PCR_TRANSFORM_DOUBLE_FLOAT, fb->keys, acc,
                                                 eps_num, eps_den, fb->status, sm_count(fb->device), s, fb->tuning,
                                                 band ? fb->band_mask : nullptr,
-                                                fb->tuning.band_bounds ? bounds_buffer(fb, s) : nullptr);
+                                                fb->tuning.band_bounds ? bounds_buffer(fb, s) : nullptr, own_pass1);
   return after_launch("k_hq_certified", (uint64_t)launched);
 }
 
@@ -411,7 +412,7 @@ pcr_status pcr_autotune(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t
       cudaEventRecord(e0, s);
       st = hq && fb->tuning.band_filter ? launch_raster_band(fb, d_points, n, dv, view->transform, 1, 100, s)
                                         : launch_raster(fb, d_points, n, dv, view->transform, s);
-      if (st == PCR_OK && hq) st = launch_hq(fb, d_points, n, dv, view->transform, 1, 100, s);
+      if (st == PCR_OK && hq) st = launch_hq(fb, d_points, n, dv, view->transform, 1, 100, s, true);
       cudaEventRecord(e1, s);
       if (cudaEventSynchronize(e1) != cudaSuccess) st = cuda_fail(cudaGetLastError(), "autotune timing");
       float ms = 0.f;
@@ -549,7 +550,7 @@ pcr_status pcr_render_hq_splat(pcr_framebuffer* fb, const pcr_point* d_points, u
                                                                     eps_den, s)
                                                : launch_raster(fb, d_points, n, dv, view->transform, s);
   if (st != PCR_OK) return st;
-  return launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, s);
+  return launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, s, true);
 }
 
 pcr_status pcr_hq_accumulate(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr_view* view,
@@ -557,7 +558,7 @@ pcr_status pcr_hq_accumulate(pcr_framebuffer* fb, const pcr_point* d_points, uin
   pcr::DevView dv;
   if (pcr_status st = check_hq(fb, d_points, n, view, eps_num, eps_den, &dv)) return st;
   if (n == 0) return PCR_OK;
-  return launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, (cudaStream_t)stream);
+  return launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, (cudaStream_t)stream, false);
 }
 
 pcr_status pcr_resolve(pcr_framebuffer* fb, uint32_t* d_rgba_out, uint32_t background_rgba, int32_t clear_after,
@@ -698,7 +699,7 @@ pcr_status pcr_render_frame_host(pcr_framebuffer* fb, const pcr_point* h_points,
     fb->band_den = eps_den;
   }
   if (hq && n > 0)
-    if (pcr_status st = launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, s)) return st;
+    if (pcr_status st = launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, s, true)) return st;
   const uint64_t npx = (uint64_t)fb->width * fb->height;
   if (pcr_status st = hq ? pcr_resolve_both(fb, d_images, d_images + npx, background_rgba, 1, stream)
                          : pcr_resolve_basic(fb, d_images, background_rgba, 1, stream))

@@ -243,8 +243,7 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
           defer = f.state >= kAmbiguous;  // undecided pixel, or code undecided between two neighbours: tier 2
         }
         commit_min<kMerge>(has && key < stored_key(keys, pix), pix, key, keys, lane, seg);
-        unsigned dummy = 0;
-        defer_points(defer, p, q, qn, lane, [&](const uint4& d) { raster_deferred(Pg, sF, d, keys, &dummy); });
+        defer_points(defer, p, q, qn, lane, [&](const uint4& d) { raster_deferred(Pg, sF, d, keys); });
       } else {
         bool accept = false;
         uint32_t pix = 0;
@@ -280,8 +279,7 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
     // the queue holds points of this view only: finish them before the next item
     if (lane < qn) {
       if (!kHq) {
-        unsigned dummy = 0;
-        raster_deferred(Pg, sF, q[lane], keys, &dummy);
+        raster_deferred(Pg, sF, q[lane], keys);
       } else {
         hq_deferred(Pg, sF, q[lane], keys, accum, eps_num, eps_den);
       }

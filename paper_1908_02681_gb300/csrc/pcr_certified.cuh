@@ -80,7 +80,7 @@ __host__ __device__ __forceinline__ bool depth_entry(const DepthColumn& c, int e
 // 1.9 KB), so concurrent launches with different views share nothing. The depth tables (12 KB a view or PIECEWISE
 // range) are not in it: every block builds them from the columns below (build_tables). They used to be built on the
 // host (14 us a view), copied to the device and read by each block: a frame with a new camera over 40,000 points took
-// 37 us that way and takes 26 us now, 1M points at 640x480 36 us and now 23 us.
+// 37 us that way and takes 26 us now, 1M points at 640x480 38 us and now 30 us.
 struct CertParams {
   // hot scalars first: the per-point loops read them as instruction operands; the columns come last
   float H[3][4], L[3][4];             // float splits of the rows clip x, clip y, w (H: nearest float, L: rest)
@@ -630,6 +630,90 @@ __device__ __forceinline__ unsigned long long code_from_fixed(uint32_t a1, uint3
   return ((unsigned long long)(a2 >> 8) << 32) | __funnelshift_r(a1, a2, 8);
 }
 
+// The fixed-point depth of a point: t * 2^40 as three 32-bit words (low first) and the top 23 fraction bits of t as a
+// float in [0, 1).
+struct FixedCode {
+  uint32_t a0, a1, a2;
+  float frac;
+};
+
+// t * 2^40 = sum m_j F_j + B (B = BH 2^32 + BL), accumulated as sum m_j F_lo_j + 2^32 sum m_j F_hi_j.
+__device__ __forceinline__ FixedCode fixed_code(const long long* __restrict__ F, const uint4& p, unsigned long long BL,
+                                                long long BH) {
+  const long long fx_ = F[p.x >> 23], fy_ = F[kTableEntries + (p.y >> 23)], fz_ = F[2 * kTableEntries + (p.z >> 23)];
+  const uint32_t mx = (p.x & 0x7FFFFFu) | 0x800000u, my = (p.y & 0x7FFFFFu) | 0x800000u,
+                 mz = (p.z & 0x7FFFFFu) | 0x800000u;
+  unsigned long long L = BL;
+  L += (unsigned long long)mx * (uint32_t)fx_;
+  L += (unsigned long long)my * (uint32_t)fy_;
+  L += (unsigned long long)mz * (uint32_t)fz_;
+  long long Hh = BH;
+  Hh += (long long)(int32_t)mx * (long long)(int32_t)(fx_ >> 32);
+  Hh += (long long)(int32_t)my * (long long)(int32_t)(fy_ >> 32);
+  Hh += (long long)(int32_t)mz * (long long)(int32_t)(fz_ >> 32);
+  FixedCode out;
+  out.a0 = (uint32_t)L;
+  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, 0;"
+      : "=r"(out.a1), "=r"(out.a2)
+      : "r"((uint32_t)(L >> 32)), "r"((uint32_t)Hh), "r"((uint32_t)((unsigned long long)Hh >> 32)));
+  out.frac = __fsub_rn(__uint_as_float(0x3F800000u | (__funnelshift_r(out.a0, out.a1, 17) & 0x7FFFFFu)), 1.0f);
+  return out;
+}
+
+// Tier 1's pixel: the estimate fm = fx - 1/2 of both axes, 1 / w, the pixel, and whether it is certain.
+struct PixelEstimate {
+  float fxm, fym, r;
+  uint32_t pixel;
+  bool ok;
+};
+
+// gx = w (fx - 1/2), gy = w (fy - 1/2) up to the rounding bounds; with wf > 0 (the depth window) fm = g * rcp(wf) and
+// the bound hE = RN(he0 - (ke s + ke3) rcp(wf)) <= 1/2 - E - 2^-25.
+template <typename PP>
+__device__ __forceinline__ PixelEstimate pixel_estimate(const PP& P, float x, float y, float z, float s, float w) {
+  PixelEstimate e;
+  const float gx = __fmaf_rn(P.Gx[2], z, __fmaf_rn(P.Gx[1], y, __fmaf_rn(P.Gx[0], x, P.Gx[3])));
+  const float gy = __fmaf_rn(P.Gy[2], z, __fmaf_rn(P.Gy[1], y, __fmaf_rn(P.Gy[0], x, P.Gy[3])));
+  e.r = rcp_approx(w);
+  e.fxm = __fmul_rn(gx, e.r);
+  e.fym = __fmul_rn(gy, e.r);
+  const float hE = __fmaf_rn(-__fmaf_rn(P.ke, s, P.ke3), e.r, P.he0);
+  // floor of fx = fm + 1/2 via the 1.5 * 2^23 shift: for -1/2 <= fm < 2^22 the sum lies in [2^23, 2^24), where
+  // floats are the integers, so g rounds fm to the nearest integer k: floor(fx) unless fx is an integer (then
+  // fx - 1 or fx, and |fm - k| = 1/2 fails the test below). Outside that range k, read from the bits, is
+  // negative or above 2^22 as an unsigned number: never below the image size.
+  const float gxx = __fadd_rn(e.fxm, 12582912.0f), gyy = __fadd_rn(e.fym, 12582912.0f);
+  const uint32_t kx = (uint32_t)(__float_as_int(gxx) - 0x4B400000), ky = (uint32_t)(__float_as_int(gyy) - 0x4B400000);
+  // fm - k = fr - 1/2 (fr = fx - k), exact (k is an integer within 1/2 of fm, both below 2^22)
+  const float dx = __fsub_rn(e.fxm, __fsub_rn(gxx, 12582912.0f)), dy = __fsub_rn(e.fym, __fsub_rn(gyy, 12582912.0f));
+  // E < fr < 1 - E for both axes: |fm - k| < hE < 1/2 - E (hE > 0 also bounds b below 1 / (2M + 1), which the
+  // bound E assumes)
+  e.ok = (kx < (uint32_t)P.v.width) & (ky < (uint32_t)P.v.height) & (fabsf(dx) < hE) & (fabsf(dy) < hE);
+  e.pixel = ky * (uint32_t)P.v.width + kx;
+  return e;
+}
+
+// Whether a point that tier 1 did not certify visible is certainly culled.
+template <typename PP>
+__device__ __forceinline__ bool certainly_culled(const PP& P, float s, float w, bool in_range, bool depth_in,
+                                                 const PixelEstimate& e) {
+  // By depth: w_d <= wf + Delta < near, or w_d >= wf - Delta >= far (directed roundings).
+  const float dw = __fmaf_rn(P.kw, s, P.kw3);
+  const bool depth_out = (__fadd_ru(w, dw) < P.near_o) | (__fsub_rd(w, dw) >= P.far_o);
+  // By the pixel, for a point inside the depth window (wf > 0): b, g from the magnitude sums, and the bound
+  // E <= |fm| (9.8u + 1.35 b) + 1.35 g + ce, valid at any |fm| while b <= 1/4.
+  const float bf = __fmul_rn(__fmul_rn(__fmaf_rn(P.Mw, s, P.Mw3), e.r), P.cb);
+  const float gf = __fmul_rn(__fmul_rn(__fmaf_rn(P.MH, s, P.MH3), e.r), P.cb);
+  const float ea = __fmaf_rn(1.35f, bf, 9.8f * 0x1p-24f), eb = __fmaf_rn(1.35f, gf, P.ce);
+  const float ex = __fmaf_rn(fabsf(e.fxm), ea, eb), ey = __fmaf_rn(fabsf(e.fym), ea, eb);
+  // fx_d < 0 when fm + 1/2 + E < 0; fx_d >= W when fm + 1/2 - E >= W (for finite bounds: an overflow leaves
+  // the point to tier 2)
+  const bool ax_out = (e.fxm < -__fadd_ru(0.5f, ex)) | (e.fxm >= __fadd_ru(P.wm, ex)) |
+                      (e.fym < -__fadd_ru(0.5f, ey)) | (e.fym >= __fadd_ru(P.hm, ey));
+  const bool e_finite = __fadd_rn(ex, ey) < 3.0e38f;
+  return in_range & (depth_out | (depth_in & (bf <= 0.25f) & e_finite & ax_out));
+}
+
 // Tier 1: the exact depth code from the fixed-point row (two 64-bit multiply-add accumulators), the cull
 // from the float w estimate and its bound, and a float pixel estimate with a rigorous per-point bound (the
 // constants and their derivation: tier1_constants). All bounds share one magnitude sum s = |x| + |y| + |z|;
@@ -691,25 +775,12 @@ __device__ __forceinline__ FastFrag classify_fast(const PP& P, const long long* 
     kd = P.kd;
     hd0 = P.hd0;
   }
-  // ---- depth code: t * 2^40 = sum m_j F_j + B, accumulated as sum m_j F_lo_j + 2^32 sum m_j F_hi_j
-  const long long fx_ = F[p.x >> 23], fy_ = F[kTableEntries + (p.y >> 23)], fz_ = F[2 * kTableEntries + (p.z >> 23)];
-  const uint32_t mx = (p.x & 0x7FFFFFu) | 0x800000u, my = (p.y & 0x7FFFFFu) | 0x800000u,
-                 mz = (p.z & 0x7FFFFFu) | 0x800000u;
-  unsigned long long L = BL;
-  L += (unsigned long long)mx * (uint32_t)fx_;
-  L += (unsigned long long)my * (uint32_t)fy_;
-  L += (unsigned long long)mz * (uint32_t)fz_;
-  long long Hh = BH;
-  Hh += (long long)(int32_t)mx * (long long)(int32_t)(fx_ >> 32);
-  Hh += (long long)(int32_t)my * (long long)(int32_t)(fy_ >> 32);
-  Hh += (long long)(int32_t)mz * (long long)(int32_t)(fz_ >> 32);
+  const FixedCode c = fixed_code(F, p, BL, BH);
+  const float frac = c.frac;
   FastFrag out;
-  out.a0 = (uint32_t)L;
-  asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, 0;"
-      : "=r"(out.a1), "=r"(out.a2)
-      : "r"((uint32_t)(L >> 32)), "r"((uint32_t)Hh), "r"((uint32_t)((unsigned long long)Hh >> 32)));
-  const float frac =
-      __fsub_rn(__uint_as_float(0x3F800000u | (__funnelshift_r(out.a0, out.a1, 17) & 0x7FFFFFu)), 1.0f);
+  out.a0 = c.a0;
+  out.a1 = c.a1;
+  out.a2 = c.a2;
   // The code is floor(t_FP64) when D < frac_exact < 1 - D, D <= kd s + d0 (the FP64 rounding and the
   // fixed-point sum's error). frac is the fraction truncated to 23 bits (frac <= frac_exact < frac + 2^-23).
   // hD = RN(hd0 - kd s), hd0 = RD(1/2 - d0 - 2^-22), is within 2^-25 of its real value, so |frac - 1/2| < hD
@@ -719,46 +790,14 @@ __device__ __forceinline__ FastFrag classify_fast(const PP& P, const long long* 
   const bool exact = fabsf(__fsub_rn(frac, 0.5f)) < hD;
   const bool amb_ok = hD > 0.25f;
 
-  // ---- pixel estimate: gx = w (fx - 1/2), gy = w (fy - 1/2) up to the rounding bounds; with wf > 0 (depth_in)
-  // fm = g * rcp(wf) and the bound hE = RN(he0 - (ke s + ke3) rcp(wf)) <= 1/2 - E - 2^-25
-  const float gx = __fmaf_rn(P.Gx[2], z, __fmaf_rn(P.Gx[1], y, __fmaf_rn(P.Gx[0], x, P.Gx[3])));
-  const float gy = __fmaf_rn(P.Gy[2], z, __fmaf_rn(P.Gy[1], y, __fmaf_rn(P.Gy[0], x, P.Gy[3])));
-  const float r = rcp_approx(w);
-  const float fxm = __fmul_rn(gx, r), fym = __fmul_rn(gy, r);
-  const float hE = __fmaf_rn(-__fmaf_rn(P.ke, s, P.ke3), r, P.he0);
-  // floor of fx = fm + 1/2 via the 1.5 * 2^23 shift: for -1/2 <= fm < 2^22 the sum lies in [2^23, 2^24), where
-  // floats are the integers, so g rounds fm to the nearest integer k: floor(fx) unless fx is an integer (then
-  // fx - 1 or fx, and |fm - k| = 1/2 fails the test below). Outside that range k, read from the bits, is
-  // negative or above 2^22 as an unsigned number: never below the image size.
-  const float gxx = __fadd_rn(fxm, 12582912.0f), gyy = __fadd_rn(fym, 12582912.0f);
-  const uint32_t kx = (uint32_t)(__float_as_int(gxx) - 0x4B400000), ky = (uint32_t)(__float_as_int(gyy) - 0x4B400000);
-  // fm - k = fr - 1/2 (fr = fx - k), exact (k is an integer within 1/2 of fm, both below 2^22)
-  const float dx = __fsub_rn(fxm, __fsub_rn(gxx, 12582912.0f)), dy = __fsub_rn(fym, __fsub_rn(gyy, 12582912.0f));
-  // E < fr < 1 - E for both axes: |fm - k| < hE < 1/2 - E (hE > 0 also bounds b below 1 / (2M + 1), which the
-  // bound E assumes)
-  const bool ax_ok = (kx < (uint32_t)P.v.width) & (ky < (uint32_t)P.v.height) & (fabsf(dx) < hE) & (fabsf(dy) < hE);
+  const PixelEstimate e = pixel_estimate(P, x, y, z, s, w);
   uint32_t st;
-  if (in_range & depth_in & ax_ok & (exact | amb_ok)) {
+  if (in_range & depth_in & e.ok & (exact | amb_ok))
     st = exact ? kExact : kAmbiguous;
-  } else {
-    // Certainly culled? By depth: w_d <= wf + Delta < near, or w_d >= wf - Delta >= far (directed roundings).
-    const float dw = __fmaf_rn(P.kw, s, P.kw3);
-    const bool depth_out = (__fadd_ru(w, dw) < P.near_o) | (__fsub_rd(w, dw) >= P.far_o);
-    // By the pixel, for a point inside the depth window (wf > 0): b, g from the magnitude sums, and the bound
-    // E <= |fm| (9.8u + 1.35 b) + 1.35 g + ce, valid at any |fm| while b <= 1/4.
-    const float bf = __fmul_rn(__fmul_rn(__fmaf_rn(P.Mw, s, P.Mw3), r), P.cb);
-    const float gf = __fmul_rn(__fmul_rn(__fmaf_rn(P.MH, s, P.MH3), r), P.cb);
-    const float ea = __fmaf_rn(1.35f, bf, 9.8f * 0x1p-24f), eb = __fmaf_rn(1.35f, gf, P.ce);
-    const float ex = __fmaf_rn(fabsf(fxm), ea, eb), ey = __fmaf_rn(fabsf(fym), ea, eb);
-    // fx_d < 0 when fm + 1/2 + E < 0; fx_d >= W when fm + 1/2 - E >= W (for finite bounds: an overflow leaves
-    // the point to tier 2)
-    const bool ax_out = (fxm < -__fadd_ru(0.5f, ex)) | (fxm >= __fadd_ru(P.wm, ex)) | (fym < -__fadd_ru(0.5f, ey)) |
-                        (fym >= __fadd_ru(P.hm, ey));
-    const bool e_finite = __fadd_rn(ex, ey) < 3.0e38f;
-    st = in_range & (depth_out | (depth_in & (bf <= 0.25f) & e_finite & ax_out)) ? kCulled : kDefer;
-  }
+  else
+    st = certainly_culled(P, s, w, in_range, depth_in, e) ? kCulled : kDefer;
   out.state = st;
-  out.pixel = ky * (uint32_t)P.v.width + kx;
+  out.pixel = e.pixel;
   return out;
 }
 
@@ -1003,17 +1042,18 @@ __device__ __forceinline__ bool raster_commit(const CertFrag& f, uint32_t rgba, 
 }
 
 // Tier 2 + arbiter for one deferred point (pass 1). Kept out of line: it runs for a small fraction of the
-// points, and inlining it would raise the register count of the main loop.
-__device__ __noinline__ void raster_deferred(const CertParams& P, const long long* sF, uint4 p,
-                                             unsigned long long* keys, unsigned* c_fp64) {
+// points, and inlining it would raise the register count of the main loop. Returns 1 when the arbiter ran.
+__device__ __noinline__ uint32_t raster_deferred(const CertParams& P, const long long* sF, uint4 p,
+                                                 unsigned long long* keys) {
   const CertFrag f = classify_cert(P, sF, p);
-  if (raster_commit(f, p.w, keys)) {
-    ++*c_fp64;
+  const bool fp64 = raster_commit(f, p.w, keys);
+  if (fp64) {
     uint32_t pix;
     unsigned long long q;
     if (project_fp64(P.v, __uint_as_float(p.x), __uint_as_float(p.y), __uint_as_float(p.z), &pix, &q))
       atomicMin(keys + pix, make_key(q, p.w));
   }
+  return fp64 ? 1u : 0u;
 }
 
 // The key a pixel holds, read through L1 (ld.global.ca). Pass 1 reads it before its atomic and skips the atomic
@@ -1176,7 +1216,7 @@ __global__ void __launch_bounds__(kCertThreads, kApprox ? PCR_CERT_APPROX_MIN_BL
       need |= has && !(kh >= bound);
     }
     if (!kApprox)
-      defer_points(defer, p, q, qn, lane, [&](const uint4& d) { raster_deferred(P, sF, d, keys, &c_fp64); });
+      defer_points(defer, p, q, qn, lane, [&](const uint4& d) { c_fp64 += raster_deferred(P, sF, d, keys); });
     return need;
   };
   const bool done = stream_tiles<kRing>(pts, n, ring[warp], bars[warp], lane,
@@ -1190,7 +1230,7 @@ __global__ void __launch_bounds__(kCertThreads, kApprox ? PCR_CERT_APPROX_MIN_BL
                                    }
                                  });
   if (!done && lane == 0) atomicOr(status, kStatusTimeout);
-  if (!kApprox && lane < qn) raster_deferred(P, sF, q[lane], keys, &c_fp64);
+  if (!kApprox && lane < qn) c_fp64 += raster_deferred(P, sF, q[lane], keys);
   if (kStats) {
     atomicAdd(stats + 0, (unsigned long long)c_exact);
     atomicAdd(stats + 1, (unsigned long long)c_amb);
@@ -1559,6 +1599,9 @@ inline void raster_launch(const uint4* pts, uint64_t n, const CertParams& P, uns
             : raster_launch4<kApprox, kMerge, false, false>(pts, n, P, keys, nullptr, status, sms, per_sm, s, band);
 }
 
+// Depth tables of prepared constants.
+inline int table_blocks(const CertParams& P) { return P.n_pw > 0 ? P.n_pw : 1; }
+
 // The certified constants of a view, prepared on this thread and kept for the next call with the same view
 // and mode. Returns false when the view is outside the single-precision preconditions.
 inline bool cached_cert(const DevView& v, bool approximate, const CertParams** out) {
@@ -1573,29 +1616,6 @@ inline bool cached_cert(const DevView& v, bool approximate, const CertParams** o
   }
   *out = &P;
   return last_ok;
-}
-
-// Pass 1 for a view with n >= 1 points. status: the framebuffer's status word (timeout bit).
-// band (mask non-null): also write the band mask for pass 2 (used only with the exact transform on LINEAR or
-// METRIC views; the caller checks that before relying on it).
-inline bool launch_raster_certified(const uint4* pts, uint64_t n, const DevView& v, bool approximate,
-                                    unsigned long long* keys, uint32_t* status, int sms, cudaStream_t s,
-                                    unsigned long long* stats = nullptr, const Tuning& t = Tuning(),
-                                    BandMask band = BandMask{nullptr, 1u, 0u, 0ull}) {
-  const CertParams* Pp = nullptr;
-  const unsigned grid = cert_grid(n, sms, t.blocks_per_sm);
-  if (!cached_cert(v, approximate, &Pp)) {
-    k_raster_fp64<<<grid, 256, 0, s>>>(pts, n, v, keys);
-    return true;
-  }
-  const int b = t.blocks_per_sm, g = t.staging;
-  if (approximate)
-    t.merge ? raster_launch<true, true>(pts, n, *Pp, keys, stats, status, sms, b, s, g)
-            : raster_launch<true, false>(pts, n, *Pp, keys, stats, status, sms, b, s, g);
-  else
-    t.merge ? raster_launch<false, true>(pts, n, *Pp, keys, stats, status, sms, b, s, g, band)
-            : raster_launch<false, false>(pts, n, *Pp, keys, stats, status, sms, b, s, g, band);
-  return true;
 }
 
 template <bool kApprox, bool kMerge, bool kRing, bool kBand = false>
@@ -1628,40 +1648,6 @@ inline void hq_launch(const uint4* pts, uint64_t n, const CertParams& P, const u
                                               nullptr, bounds)
           : hq_launch4<kApprox, kMerge, false>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s,
                                                nullptr, bounds);
-}
-
-// Pass 2 for a view with n >= 1 points. status: the framebuffer's status word (timeout bit). band_mask: see
-// hq_launch. bounds_buf: room for the accept bounds of every pixel (npx entries), or null; with the exact
-// transform and band_bounds_exact they are computed (k_band_bounds) and pass 2 tests against them. Returns the
-// number of kernels launched.
-inline int launch_hq_certified(const uint4* pts, uint64_t n, const DevView& v, bool approximate,
-                               const unsigned long long* keys, unsigned long long* accum, uint32_t eps_num,
-                               uint32_t eps_den, uint32_t* status, int sms, cudaStream_t s,
-                               const Tuning& t = Tuning(), const uint32_t* band_mask = nullptr, ulonglong2* bounds_buf = nullptr) {
-  const CertParams* Pp = nullptr;
-  const unsigned grid = cert_grid(n, sms, t.blocks_per_sm);
-  if (!cached_cert(v, approximate, &Pp) || Pp->n_pw > 0) {  // (HQ takes LINEAR or METRIC views only)
-    k_hq_fp64<<<grid, 256, 0, s>>>(pts, n, v, keys, accum, eps_num, eps_den);
-    return 1;
-  }
-  const int b = t.blocks_per_sm, g = t.staging;
-  if (approximate) {
-    t.merge ? hq_launch<true, true>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g)
-            : hq_launch<true, false>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g);
-    return 1;
-  }
-  const ulonglong2* bounds = nullptr;
-  if (bounds_buf && band_bounds_exact(v.nq, eps_num, eps_den)) {
-    const uint64_t npx = (uint64_t)v.width * v.height;
-    const unsigned bgrid = (unsigned)((npx + 255) / 256 < (uint64_t)sms * 8 ? (npx + 255) / 256 : (uint64_t)sms * 8);
-    k_band_bounds<<<bgrid, 256, 0, s>>>(keys, npx, v.nq, eps_num, div_magic(eps_den), bounds_buf);
-    bounds = bounds_buf;
-  }
-  t.merge ? hq_launch<false, true>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g,
-                                   band_mask, bounds)
-          : hq_launch<false, false>(pts, n, *Pp, keys, accum, eps_num, eps_den, status, sms, b, s, g,
-                                    band_mask, bounds);
-  return bounds ? 2 : 1;
 }
 
 }  // namespace pcr

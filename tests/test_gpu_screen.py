@@ -1,0 +1,108 @@
+"""The screened passes (csrc/pcr_screen.cuh), which the exact transform runs with default tuning on LINEAR and METRIC
+views, against the FP64 kernels, bit for bit: sizes at the edges of tiles, warps and blocks, dense runs on one pixel,
+codes next to the stored one and to the band's edges, bands the screen leaves to k_hq_cert, keys left by another depth
+mapping or another cloud."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import scenes
+from tests.helpers import RawView, axis_view, pack
+
+pytestmark = pytest.mark.gpu
+
+
+def _dev(points):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(points).view(np.int32)).cuda()
+
+
+def _view(v, depth=0, scale=1000.0, transform=0):
+    return RawView(np.asarray(v.view_proj), v.near, v.far, v.width, v.height, depth, scale, None, transform)
+
+
+def _frames(gpu, dev, v, depth, scale, eps, before=None, accumulate=False, tuning=None):
+    """Keys and sums of one frame by the exact and by the FP64 transform."""
+    res = []
+    for transform in (0, 1):
+        fb = gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ)
+        if tuning and transform == 0:
+            gpu.pcr_set_tuning(fb, **tuning)
+        view = _view(v, depth, scale, transform)
+        if before:
+            before(fb)
+        if accumulate:
+            gpu.pcr_hq_accumulate(fb, dev, view, *eps)
+        else:
+            gpu.pcr_render_hq_splat(fb, dev, view, *eps)
+        keys, acc = gpu.pcr_framebuffer_keys(fb)
+        res.append((keys.clone(), acc.clone()))
+        assert gpu.pcr_get_device_status(fb) == gpu.PCR_OK
+        fb.close()
+    assert int((res[0][0] != res[1][0]).sum()) == 0
+    assert int((res[0][1] != res[1][1]).sum()) == 0
+    return res[0]
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 63, 64, 65, 127, 129, 2047, 2048, 2049, 38911, 38913, 152 * 2048 + 1, 700001])
+def test_sizes(gpu, n):
+    v = scenes.lidar_1km_view(320, 180)
+    keys, _ = _frames(gpu, _dev(scenes.lidar(n, 41)), v, 0, 1.0, (1, 100))
+    assert int((keys != -1).sum()) > 0 or n < 64
+
+
+@pytest.mark.parametrize("depth,scale", [(0, 1.0), (1, 1000.0), (1, 1e6), (1, 1e8)])
+@pytest.mark.parametrize("eps", [(1, 100), (0, 1), (3, 1), (1, 1 << 20), (1 << 20, 1), (16_000_000, 1 << 20)])
+def test_depth_modes_and_bands(gpu, depth, scale, eps):
+    v = scenes.lidar_1km_view(160, 90)
+    pts = scenes.lidar(400_001, 42)
+    scenes.shuffle(pts, 3)
+    _frames(gpu, _dev(pts), v, depth, scale, eps)
+
+
+@pytest.mark.parametrize("spread", [0.0, 1e-7, 1e-6, 1e-4, 1e-2])
+@pytest.mark.parametrize("eps", [(1, 100), (1, 1 << 20), (0, 1)])
+def test_codes_next_to_the_stored_one(gpu, spread, eps):
+    """Many points on few pixels in one depth sheet: codes from equal to a few units apart, in runs and shuffled."""
+    rng = np.random.default_rng(7)
+    n = 100_000
+    w = 3.0 * (1.0 + spread * rng.random(n))
+    ndc = np.repeat(rng.uniform(-0.9, 0.9, (n // 50, 2)), 50, axis=0) + rng.uniform(0, 1e-3, (n, 2))
+    pts = pack(np.column_stack([ndc[:, 0] * w, ndc[:, 1] * w, -w]), rng.integers(0, 1 << 32, n, dtype=np.uint64))
+    for _ in range(2):
+        _frames(gpu, _dev(pts), axis_view(64, 48), 0, 1.0, eps)
+        rng.shuffle(pts)
+
+
+def test_one_pixel_and_every_tuned_grid(gpu):
+    rng = np.random.default_rng(8)
+    w = rng.uniform(1.0, 8.0, 300_000)
+    pts = _dev(pack(np.column_stack([0.01 * w, 0.01 * w, -w]), np.arange(300_000, dtype=np.uint32)))
+    for blocks in (1, 2, 3, 8, 32):
+        _frames(gpu, pts, axis_view(64, 48), 0, 1.0, (1, 10), tuning={"blocks_per_sm": blocks})
+
+
+@pytest.mark.parametrize("depth,scale", [(0, 1.0), (1, 1000.0), (1, 1e8)])
+def test_keys_of_another_mapping_and_cloud(gpu, depth, scale):
+    """A frame on keys that a LINEAR view and another cloud left (larger and smaller codes than the frame's own), and
+    pass 2 alone on such keys (points in front of their pixel's key are outside the band) and on an empty framebuffer."""
+    v = scenes.lidar_1km_view(200, 120)
+    other, dev = _dev(scenes.lidar(50_000, 44)), _dev(scenes.lidar(300_000, 45))
+
+    def before(fb):
+        gpu.pcr_render_atomicmin(fb, other, _view(v, 0))
+
+    _frames(gpu, dev, v, depth, scale, (1, 100), before)
+    _frames(gpu, dev, v, depth, scale, (1, 100), before, accumulate=True)
+    _frames(gpu, dev, v, depth, scale, (1, 100), accumulate=True)
+
+
+def test_special_coordinates(gpu):
+    pts = scenes.lidar(200_000, 46)
+    f = pts[:, :3].view(np.float32)
+    rng = np.random.default_rng(9)
+    for value in (np.nan, np.inf, -np.inf, 3e38, -3e38, 1e20, 1e-42, 0.0, -0.0):
+        f[rng.integers(0, len(pts), 800), rng.integers(0, 3, 800)] = value
+    for depth, scale in ((0, 1.0), (1, 1000.0)):
+        _frames(gpu, _dev(pts), scenes.lidar_1km_view(320, 180), depth, scale, (1, 100))
