@@ -329,50 +329,67 @@ inline int batch_pass_resident(const BatchTuning& t) {
   return b;
 }
 
-// Resolve of every framebuffer of a batch (pcr_resolve semantics per view), one launch. pixel_start[v] =
-// first global pixel of view v, pixel_start[n_views] = total.
-__global__ void __launch_bounds__(256) k_resolve_batch(const BatchSlot* __restrict__ slots,
-                                                       const uint64_t* __restrict__ pixel_start, uint32_t n_views,
-                                                       uint32_t background, int clear) {
-  const uint64_t total = pixel_start[n_views];
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-    uint32_t v = 0;
-    uint32_t lo = 0, hi = n_views;  // last v with pixel_start[v] <= g
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (pixel_start[mid] <= g) lo = mid; else hi = mid;
+// Resolve of every framebuffer of a batch (pcr_resolve semantics per view), one launch: blockIdx.y is the view, whose
+// pixels the view's blocks take kResolveStep pixels a thread at a time, so that every thread has several independent
+// 16-byte loads in flight and no pixel looks its view up. Bound by DRAM (the framebuffers of a batch exceed L2): 20
+// bytes a pixel read and written with a clear, 44 with high-quality sums. On one GB300, 16 views of mixed sizes (53.7M
+// pixels, basic): 325 us with one pixel a thread and a binary search for its view, 152 us now; 12 views
+// (42.7M pixels) high-quality: 386 and 270 us.
+constexpr int kResolveStep = 4;
+
+__global__ void __launch_bounds__(256) k_resolve_batch(const BatchSlot* __restrict__ slots, uint32_t background, int clear) {
+  const BatchSlot& S = slots[blockIdx.y];
+  const uint64_t npx = (uint64_t)S.width * S.height;
+  unsigned long long* const keys = S.keys;
+  ulonglong2* const acc = reinterpret_cast<ulonglong2*>(S.accum);
+  uint32_t* const out = S.out;
+  const uint64_t stride = (uint64_t)gridDim.x * (256 * kResolveStep);
+  uint64_t i0 = (uint64_t)blockIdx.x * (256 * kResolveStep) + threadIdx.x;
+  if (S.hq) {
+    bool overflow = false;
+    for (; i0 < npx; i0 += stride) {
+      ulonglong2 a[kResolveStep];
+#pragma unroll
+      for (int k = 0; k < kResolveStep; ++k)
+        if (i0 + 256 * k < npx) a[k] = acc[i0 + 256 * k];
+#pragma unroll
+      for (int k = 0; k < kResolveStep; ++k) {
+        const uint64_t i = i0 + 256 * k;
+        if (i >= npx) break;
+        out[i] = hq_colour(a[k], background, overflow);
+        if (clear) {
+          acc[i] = make_ulonglong2(0ull, 0ull);
+          keys[i] = kEmptyKey;
+        }
+      }
     }
-    v = lo;
-    const BatchSlot& S = slots[v];
-    const uint64_t i = g - pixel_start[v];
-    unsigned long long* keys = S.keys;
-    ulonglong2* acc = reinterpret_cast<ulonglong2*>(S.accum);
-    if (S.hq) {
-      const ulonglong2 a = acc[i];
-      const uint32_t c = (uint32_t)(a.y >> 32);
-      if (c == 0) {
-        S.out[i] = background;
-      } else {
-        if (c > (1u << 24)) atomicOr(S.status, kStatusOverflow);
-        const uint32_t r = (uint32_t)(((a.x & 0xFFFFFFFFull) + c / 2) / c);
-        const uint32_t gg = (uint32_t)(((a.x >> 32) + c / 2) / c);
-        const uint32_t b = (uint32_t)(((a.y & 0xFFFFFFFFull) + c / 2) / c);
-        S.out[i] = (r & 0xFFu) | ((gg & 0xFFu) << 8) | ((b & 0xFFu) << 16) | 0xFF000000u;
-      }
-      if (clear) {
-        acc[i] = make_ulonglong2(0ull, 0ull);
-        keys[i] = kEmptyKey;
-      }
-    } else {
-      const unsigned long long k = keys[i];
-      S.out[i] = k == kEmptyKey ? background : ((uint32_t)(k & 0xFFFFFFu) | 0xFF000000u);
-      if (clear) {
-        keys[i] = kEmptyKey;
-        if (acc) acc[i] = make_ulonglong2(0ull, 0ull);
+    if (overflow) atomicOr(S.status, kStatusOverflow);
+  } else {
+    for (; i0 < npx; i0 += stride) {
+      unsigned long long q[kResolveStep];
+#pragma unroll
+      for (int k = 0; k < kResolveStep; ++k)
+        if (i0 + 256 * k < npx) q[k] = keys[i0 + 256 * k];
+#pragma unroll
+      for (int k = 0; k < kResolveStep; ++k) {
+        const uint64_t i = i0 + 256 * k;
+        if (i >= npx) break;
+        out[i] = basic_colour(q[k], background);
+        if (clear) {
+          keys[i] = kEmptyKey;
+          if (acc) acc[i] = make_ulonglong2(0ull, 0ull);
+        }
       }
     }
   }
+}
+
+// The batch resolve of `count` views on a device of `sms` SMs: enough blocks a view to fill the device alone several
+// times over, no more than the largest possible view needs.
+inline void launch_resolve_batch(const BatchSlot* slots, int count, uint64_t most_pixels, uint32_t background, int clear,
+                                 int sms, cudaStream_t s) {
+  const uint64_t need = (most_pixels + 256 * kResolveStep - 1) / (256 * kResolveStep), cap = (uint64_t)sms * 8;
+  k_resolve_batch<<<dim3((unsigned)(need < cap ? need : cap), (unsigned)count), 256, 0, s>>>(slots, background, clear);
 }
 
 }  // namespace pcr

@@ -57,14 +57,39 @@ __global__ void __launch_bounds__(256) k_hq_fp64(const uint4* __restrict__ pts, 
   }
 }
 
-// Section 2.1 resolve: key -> RGBA8 (alpha 255), background where empty; optional clear (keys, and the
-// HQ sums when present).
+// Section 2.1 resolve of one key: RGBA8 with alpha 255, background where empty.
+__device__ __forceinline__ uint32_t basic_colour(unsigned long long k, uint32_t background) {
+  return k == kEmptyKey ? background : ((uint32_t)(k & 0xFFFFFFu) | 0xFF000000u);
+}
+
+// Section 2.2 average of one pixel's sums: per channel (sum + count / 2) / count, alpha 255, background where count is
+// 0. A count above 2^24 means a u32 colour sum may have wrapped: flagged (the same arithmetic as the oracle's, in 64
+// bits, then).
+__device__ __forceinline__ uint32_t hq_colour(const ulonglong2& a, uint32_t background, bool& overflow) {
+  const uint32_t c = (uint32_t)(a.y >> 32);
+  if (c == 0) return background;
+  uint32_t r, g, b;
+  if (c <= (1u << 24)) {
+    // each channel sum is at most 255 c, so sum + c / 2 < 2^32: the 32-bit quotient is the same
+    const uint32_t h = c / 2;
+    r = ((uint32_t)a.x + h) / c;
+    g = ((uint32_t)(a.x >> 32) + h) / c;
+    b = ((uint32_t)a.y + h) / c;
+  } else {
+    overflow = true;
+    r = (uint32_t)(((a.x & 0xFFFFFFFFull) + c / 2) / c);
+    g = (uint32_t)(((a.x >> 32) + c / 2) / c);
+    b = (uint32_t)(((a.y & 0xFFFFFFFFull) + c / 2) / c);
+  }
+  return (r & 0xFFu) | ((g & 0xFFu) << 8) | ((b & 0xFFu) << 16) | 0xFF000000u;
+}
+
+// Section 2.1 resolve: key -> RGBA8; optional clear (keys, and the HQ sums when present).
 __global__ void k_resolve_basic(unsigned long long* __restrict__ keys, ulonglong2* __restrict__ accum,
                                 uint32_t* __restrict__ rgba, uint64_t npx, uint32_t background, int clear) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += stride) {
-    const unsigned long long k = keys[i];
-    rgba[i] = k == kEmptyKey ? background : ((uint32_t)(k & 0xFFFFFFu) | 0xFF000000u);
+    rgba[i] = basic_colour(keys[i], background);
     if (clear) {
       keys[i] = kEmptyKey;
       if (accum) accum[i] = make_ulonglong2(0ull, 0ull);
@@ -72,32 +97,14 @@ __global__ void k_resolve_basic(unsigned long long* __restrict__ keys, ulonglong
   }
 }
 
-// Section 2.2 third pass: per channel (sum + count / 2) / count, alpha 255, background where count is 0.
-// A count above 2^24 means a u32 colour sum may have wrapped: flagged in the status word.
+// Section 2.2 third pass: the averages of the sums; the status word's overflow bit where a count is above 2^24.
 __global__ void k_resolve_hq(ulonglong2* __restrict__ accum, unsigned long long* __restrict__ keys,
                              uint32_t* __restrict__ rgba, uint64_t npx, uint32_t background, int clear,
                              uint32_t* __restrict__ status) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   bool overflow = false;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += stride) {
-    const ulonglong2 a = accum[i];
-    const uint32_t c = (uint32_t)(a.y >> 32);
-    if (c == 0) {
-      rgba[i] = background;
-    } else if (c <= (1u << 24)) {
-      // each channel sum is at most 255 c, so sum + c / 2 < 2^32: the 32-bit quotient is the same
-      const uint32_t h = c / 2;
-      const uint32_t r = ((uint32_t)a.x + h) / c;
-      const uint32_t g = ((uint32_t)(a.x >> 32) + h) / c;
-      const uint32_t b = ((uint32_t)a.y + h) / c;
-      rgba[i] = (r & 0xFFu) | ((g & 0xFFu) << 8) | ((b & 0xFFu) << 16) | 0xFF000000u;
-    } else {  // more fragments than the sums can hold: flagged; the same arithmetic as the oracle's, in 64 bits
-      overflow = true;
-      const uint32_t r = (uint32_t)(((a.x & 0xFFFFFFFFull) + c / 2) / c);
-      const uint32_t g = (uint32_t)(((a.x >> 32) + c / 2) / c);
-      const uint32_t b = (uint32_t)(((a.y & 0xFFFFFFFFull) + c / 2) / c);
-      rgba[i] = (r & 0xFFu) | ((g & 0xFFu) << 8) | ((b & 0xFFu) << 16) | 0xFF000000u;
-    }
+    rgba[i] = hq_colour(accum[i], background, overflow);
     if (clear) {
       accum[i] = make_ulonglong2(0ull, 0ull);
       keys[i] = kEmptyKey;
@@ -117,25 +124,8 @@ __global__ void k_resolve_both(unsigned long long* __restrict__ keys, ulonglong2
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += stride) {
     const unsigned long long k = keys[i];
     const ulonglong2 a = accum[i];
-    rgba_basic[i] = k == kEmptyKey ? background : ((uint32_t)(k & 0xFFFFFFu) | 0xFF000000u);
-    const uint32_t c = (uint32_t)(a.y >> 32);
-    uint32_t r, g, b;
-    if (c == 0) {
-      rgba_hq[i] = background;
-    } else {
-      if (c <= (1u << 24)) {  // as in k_resolve_hq: 32-bit quotients below the overflow bound
-        const uint32_t h = c / 2;
-        r = ((uint32_t)a.x + h) / c;
-        g = ((uint32_t)(a.x >> 32) + h) / c;
-        b = ((uint32_t)a.y + h) / c;
-      } else {
-        overflow = true;
-        r = (uint32_t)(((a.x & 0xFFFFFFFFull) + c / 2) / c);
-        g = (uint32_t)(((a.x >> 32) + c / 2) / c);
-        b = (uint32_t)(((a.y & 0xFFFFFFFFull) + c / 2) / c);
-      }
-      rgba_hq[i] = (r & 0xFFu) | ((g & 0xFFu) << 8) | ((b & 0xFFu) << 16) | 0xFF000000u;
-    }
+    rgba_basic[i] = basic_colour(k, background);
+    rgba_hq[i] = hq_colour(a, background, overflow);
     if (clear) {
       keys[i] = kEmptyKey;
       accum[i] = make_ulonglong2(0ull, 0ull);
