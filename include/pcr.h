@@ -341,7 +341,8 @@ typedef struct {
                                 of at least 10^8 points (outside graph capture), else the batch kernel; 1: always
                                 the batch kernel; 2: always one single-view pass per view */
   int32_t slice_words;       /* batch kernel work item: 1 (default), 2 or 4 words of a view's chunk mask
-                                (32, 64 or 128 chunks of 1024 points) */
+                                (32, 64 or 128 chunks of 1024 points); halved, down to one chunk, while a frame has
+                                too few items for the grid */
   int32_t points_per_thread; /* points a thread classifies per step of the batch kernel: 1 (default) or 2 */
   int32_t blocks_per_sm;     /* 256-thread blocks per SM of the batch kernel, 1..32 (default 4; capped at the
                                 blocks that can be resident) */

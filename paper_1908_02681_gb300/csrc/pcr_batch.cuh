@@ -17,7 +17,7 @@
 //   * one resolve launch for all views.
 #pragma once
 
-#include "pcr_certified.cuh"
+#include "pcr_screen.cuh"
 
 namespace pcr {
 
@@ -154,13 +154,15 @@ struct BatchTuning {
 };
 
 // Pass 1 (kHq = false) or pass 2 (kHq = true) for every view of a batch, one persistent launch. Work item
-// = (range r of slice_words consecutive mask words, i.e. 32 * slice_words chunks, view v), numbered
+// = (range r of slice_chunks consecutive chunks: 32 or a multiple or a power-of-two part of it, view v), numbered
 // r * n_views + v and taken in that order from next_item[kHq]: the views of one range run close together in
 // time, so the range's points come from HBM once and from L2 for the other views. Warp 0 lists the range's
 // chunks whose mask bit is set; the block then walks them in steps of kCertThreads * kPts points (each warp
 // takes 32 * kPts consecutive points per step), loading the next step's points before classifying the
 // current ones. params: per-view CertParams in device memory (tier 2 and the FP64 arbiter read them there;
-// tier 1 holds its constants in registers for the item). merge_width: see BatchTuning (kMerge = width > 0).
+// tier 1 holds its constants in registers for the item). merge_width: see BatchTuning (kMerge = width > 0). Without
+// merging, pass 2's accepted fragments go through the paired additions of AddQueue, finished with the item (12 views of
+// 6M points on one GB300: the frame 1.49 to 1.42 ms, against one pair of additions per lane).
 #ifndef PCR_BATCH_MIN_BLOCKS
 #define PCR_BATCH_MIN_BLOCKS 4
 #endif
@@ -168,19 +170,21 @@ template <bool kHq, bool kMerge, int kPts>
 __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pass(
     const uint4* __restrict__ pts, uint64_t n, const CertParams* __restrict__ params,
     const long long* __restrict__ tables, const BatchSlot* __restrict__ slots, const uint32_t* __restrict__ masks, uint32_t n_views, uint32_t n_chunks,
-    uint32_t* __restrict__ next_item, uint32_t eps_num, uint32_t eps_den, uint32_t slice_words,
+    uint32_t* __restrict__ next_item, uint32_t eps_num, uint32_t eps_den, uint32_t slice_chunks,
     uint32_t merge_width) {
   __shared__ long long sF[3 * kTableEntries];
   __shared__ uint4 queue[kCertWarps][kQueue];
   __shared__ uint32_t s_chunks[kMaxSliceWords * 32];
+  __shared__ __align__(16) uint2 add_ring[kHq && !kMerge ? kCertWarps : 1][kAddRing];
   __shared__ uint32_t s_item, s_nvis;
   static_assert(kPts == 1 || kPts == 2, "one or two points per thread per step");
   static_assert(kChunk % (kCertThreads * kPts) == 0, "whole steps per chunk");
   constexpr uint32_t kSteps = kChunk / (kCertThreads * kPts);  // steps per chunk
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   uint4* q = queue[warp];
+  AddQueue aq{add_ring[kHq && !kMerge ? warp : 0], 0u, 0u};
   const uint32_t words = (n_chunks + 31u) / 32u;
-  const uint32_t ranges = (words + slice_words - 1u) / slice_words;
+  const uint32_t ranges = (n_chunks + slice_chunks - 1u) / slice_chunks;
   const uint32_t total = ranges * n_views;
   const uint32_t seg = merge_segment(lane, merge_width);
   uint32_t cur_view = 0xFFFFFFFFu;
@@ -190,12 +194,13 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
     const uint32_t item = s_item;
     if (item >= total) break;
     const uint32_t r = item / n_views, v = item - r * n_views;
-    const uint32_t w0 = r * slice_words;
-    const uint32_t wn = words - w0 < slice_words ? words - w0 : slice_words;
+    const uint32_t w0 = r * slice_chunks / 32u;
+    const uint32_t last = (r + 1u) * slice_chunks < n_chunks ? (r + 1u) * slice_chunks : n_chunks;
     if (warp == 0) {  // the visible chunks of the item, in increasing order
       uint32_t cnt = 0;
-      for (uint32_t k = 0; k < wn; ++k) {
-        const uint32_t bits = masks[(uint64_t)v * words + w0 + k];
+      for (uint32_t k = 0; (w0 + k) * 32u < last; ++k) {
+        uint32_t bits = masks[(uint64_t)v * words + w0 + k];
+        if (slice_chunks < 32u) bits &= ((1u << slice_chunks) - 1u) << (r * slice_chunks % 32u);
         if ((bits >> lane) & 1u) s_chunks[cnt + __popc(bits & ((1u << lane) - 1u))] = (w0 + k) * 32u + lane;
         cnt += __popc(bits);
       }
@@ -256,8 +261,8 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
         }
         if constexpr (kMerge)
           commit_add<true>(accept, pix, p.w, accum, lane, seg);
-        else  // consecutive points in adjacent lanes: merged in lane pairs (commit_add_pairs)
-          commit_add_pairs(accept, pix, p.w, accum, lane);
+        else
+          add_push(accept, pix, p.w, aq, lane);
         defer_points(defer, p, q, qn, lane,
                      [&](const uint4& d) { hq_deferred(Pg, sF, d, keys, accum, eps_num, eps_den); });
       }
@@ -275,6 +280,14 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
       }
       point(c0, i < n);
       if (kPts == 2) point(c1, i + 32 < n);
+      if constexpr (kHq && !kMerge) add_drain_full(aq, accum, lane);
+    }
+    if constexpr (kHq && !kMerge) {  // the queued additions are this view's
+      if (aq.tail != aq.head) {
+        add_finish(aq, accum, lane);
+        aq.head += 64u;
+        aq.tail = aq.head;
+      }
     }
     // the queue holds points of this view only: finish them before the next item
     if (lane < qn) {
@@ -289,6 +302,11 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
   }
 }
 
+// Least work items per block of a batch pass: with fewer, blocks stay idle or end unevenly. On one GB300, 16 views of
+// mixed sizes: 300,000 points 0.57 to 0.28 ms against items of 32 chunks at least, 2M points 0.72 to 0.44 (1 item a
+// block: 0.49, 8: 0.46), 20M unchanged.
+constexpr int kMinItems = 4;
+
 // Launches the batch pass kernel of a tuning (template instance by merging and points per thread).
 template <bool kHq>
 inline void batch_pass_launch(const BatchTuning& t, int sms, int resident, const uint4* pts, uint64_t n,
@@ -297,10 +315,13 @@ inline void batch_pass_launch(const BatchTuning& t, int sms, int resident, const
                               uint32_t eps_den, cudaStream_t s) {
   const int per_sm = t.blocks_per_sm < resident ? t.blocks_per_sm : resident;
   const unsigned grid = (unsigned)(sms * (per_sm > 0 ? per_sm : 1));
-  const uint32_t sw = (uint32_t)t.slice_words, mw = (uint32_t)t.merge_width;
+  const uint32_t mw = (uint32_t)t.merge_width;
+  // work items of slice_words mask words (32 chunks each), halved while the frame has fewer than kMinItems a block
+  uint32_t sc = 32u * (uint32_t)t.slice_words;
+  while (sc > 1u && (uint64_t)((n_chunks + sc - 1u) / sc) * n_views < (uint64_t)kMinItems * grid) sc /= 2u;
 #define PCR_BATCH_LAUNCH(M, K)                                                                                    \
   k_batch_pass<kHq, M, K><<<grid, kCertThreads, 0, s>>>(pts, n, params, tables, slots, masks, n_views, n_chunks, \
-                                                        next_item, eps_num, eps_den, sw, mw)
+                                                        next_item, eps_num, eps_den, sc, mw)
   if (t.merge_width > 0) {
     if (t.points_per_thread == 2) PCR_BATCH_LAUNCH(true, 2); else PCR_BATCH_LAUNCH(true, 1);
   } else {
