@@ -19,8 +19,8 @@ namespace pcr {
 //   |wf - w_d| <= Delta <= 4.0005u (Mw s + Mw3), |wf| <= Mw s + Mw3 (tier1_constants), u = 2^-24. An edge
 //   e(sh) = RN(a sh + b), a and b >= 0 or a = 0, is within 3.1u |e| of its real value (roundings of sh, a, b, the fma).
 //   With the margin m(s) = RN(k s + k3) >= (Delta + c + 3.1u |wf|)(1 + 16u), c the slack below:
-//     RN(wf - e) > m   implies  w_d >= e_real + c: wf - e > m (1 - u), and e_real <= e + 3.1u e <= e + 3.1u wf
-//     RN(wf - e) < -m  implies  w_d <= e_real - c: e_real >= e - 3.1u e, and 3.1u e = 3.1u (e - wf) + 3.1u wf
+//     RN(wf - e) >= m  implies  w_d >= e_real + c: wf - e >= m (1 - u), and e_real <= e + 3.1u e <= e + 3.1u wf
+//     RN(wf - e) <= -m implies  w_d <= e_real - c: e_real >= e - 3.1u e, and 3.1u e = 3.1u (e - wf) + 3.1u wf
 //   c S covers the width of the stored code's unit and the 2^-11 of t_d.
 //   PIECEWISE (pass 1 only): codes grow with w across the ranges, so a point in range r has a larger code than qs iff it
 //   lies beyond the edge lo_r + (qs + 1 - base_r) / res_r, wherever qs itself lies. Its b = lo_r + (unit - base_r) / res_r
@@ -116,7 +116,8 @@ __device__ __forceinline__ float ranged(const float* f, int r) {
 }
 
 // Tier 1 without the depth code, of one point: what the test against its stored key needs. A point that is not
-// certainly visible has w = 3e38 (the tests of both passes drop it) and needs no key.
+// certainly visible has w = +inf, so that the ordered comparisons of both passes' tests drop it whatever its coordinates
+// (their magnitude sum, hence the margin, may be infinite or NaN) and its pixel is never used.
 struct ScreenPoint {
   uint32_t pixel;
   float w, m;  // depth estimate and margin
@@ -147,7 +148,7 @@ __device__ __forceinline__ ScreenPoint screen_point(const CertParams& P, const S
     o.k = stored_depth<kMode>(keys, o.pixel);
   } else {
     o.open = !certainly_culled(P, s, o.w, s < P.xyz_max, depth_in, e);
-    o.w = 3.0e38f;
+    o.w = __int_as_float(0x7F800000);
   }
   return o;
 }
@@ -316,8 +317,8 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
           push_open(s0.open, place, q.open, on, lane);
           push_open(s1.open, place + 32u, q.open, on, lane);
         }
-        const bool n0 = !(__fsub_rn(s0.w, __fmaf_rn(s0.k, s0.a, s0.b)) > s0.m);
-        const bool n1 = !(__fsub_rn(s1.w, __fmaf_rn(s1.k, s1.a, s1.b)) > s1.m);
+        const bool n0 = __fsub_rn(s0.w, __fmaf_rn(s0.k, s0.a, s0.b)) < s0.m;
+        const bool n1 = __fsub_rn(s1.w, __fmaf_rn(s1.k, s1.a, s1.b)) < s1.m;
         const int need = __popc(__ballot_sync(0xFFFFFFFFu, n0)) + __popc(__ballot_sync(0xFFFFFFFFu, n1));
         if (need >= kDirect) {
           commit(n0, p0, s0.pixel, place);
@@ -446,14 +447,14 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
           push_open(s0.open, place, q.open, on, lane);
           push_open(s1.open, place + 32u, q.open, on, lane);
         }
-        auto inside = [&](const ScreenPoint& o) {  // > m: in the band; < -m: outside it
+        auto inside = [&](const ScreenPoint& o) {  // >= m: in the band; <= -m: outside it
           return fminf(__fsub_rn(o.w, __fmaf_rn(o.k, S.lo_a, S.lo_b)), __fsub_rn(__fmaf_rn(o.k, S.hi_a, S.hi_b), o.w));
         };
         const float d0 = inside(s0), d1 = inside(s1);
-        add_push(d0 > s0.m, s0.pixel, p0.w, aq, lane);
-        add_push(d1 > s1.m, s1.pixel, p1.w, aq, lane);
+        add_push(d0 >= s0.m, s0.pixel, p0.w, aq, lane);
+        add_push(d1 >= s1.m, s1.pixel, p1.w, aq, lane);
         add_drain_full(aq, accum, lane);
-        const bool n0 = !(fabsf(d0) > s0.m), n1 = !(fabsf(d1) > s1.m);
+        const bool n0 = fabsf(d0) < s0.m, n1 = fabsf(d1) < s1.m;
         if (__any_sync(0xFFFFFFFFu, n0 | n1)) {
           push_candidate(n0, p0, s0.pixel, place, q, cn, lane);
           push_candidate(n1, p1, s1.pixel, place + 32u, q, cn, lane);

@@ -106,3 +106,15 @@ def test_special_coordinates(gpu):
         f[rng.integers(0, len(pts), 800), rng.integers(0, 3, 800)] = value
     for depth, scale in ((0, 1.0), (1, 1000.0)):
         _frames(gpu, _dev(pts), scenes.lidar_1km_view(320, 180), depth, scale, (1, 100))
+
+
+def test_visible_points_whose_magnitude_sum_overflows(gpu):
+    """|x| + |y| + |z| is infinite in float, yet the FP64 definition draws the point: it must count once."""
+    m = np.zeros((4, 4))
+    m[0, 0], m[0, 1], m[1, 2], m[2, 2], m[3, 2] = 1.0, -1.0, 0.25, -1.0, -1.0
+    n = 5000
+    rng = np.random.default_rng(10)
+    big = rng.uniform(2.0e38, 3.0e38, n).astype(np.float32)
+    pts = pack(np.column_stack([big, big, -rng.uniform(1.0, 8.0, n)]), rng.integers(0, 1 << 32, n, dtype=np.uint64))
+    _, acc = _frames(gpu, _dev(pts), RawView(m, 0.5, 8.5, 64, 48), 0, 1.0, (10, 1))
+    assert int((acc[:, 1] >> 32).sum()) == n

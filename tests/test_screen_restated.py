@@ -62,14 +62,14 @@ def test_decisions(depth, scale, eps):
         for d in (0, 1, -1, 255, -256, 300, -300, *(f * margin for f in (-3.0, -1.2, -0.9, -0.3, 0.3, 0.9, 1.2, 3.0))):
             qs = np.clip(centre + np.asarray(d, np.float64).astype(np.int64), 0, 2 ** 40 - 2)
             # pass 1
-            skip = (w - fma32(sc.stored(qs), sc.a, sc.b)).astype(np.float32) > m1
+            skip = (w - fma32(sc.stored(qs), sc.a, sc.b)).astype(np.float32) >= m1
             assert not (skip & (q <= qs)).any()
             # pass 2
             k = sb.stored(qs)
             dist = np.minimum((w - fma32(k, *sb.lo)).astype(np.float32), (fma32(k, *sb.hi) - w).astype(np.float32))
             band = (q >= qs) & ((q - qs).astype(object) * den <= num * (qs.astype(object) + sb.nq))
-            assert not ((dist > m2) & ~band).any()
-            assert not ((dist < -m2) & band).any()
-            for name, n in (("skip", skip), ("in", dist > m2), ("out", dist < -m2)):
+            assert not ((dist >= m2) & ~band).any()
+            assert not ((dist <= -m2) & band).any()
+            for name, n in (("skip", skip), ("in", dist >= m2), ("out", dist <= -m2)):
                 sizes[name] = sizes.get(name, 0) + int(n.sum())
     assert sizes["skip"] > 0 and sizes["out"] > 0 and (num == 0 or eps[1] > 1000 or sizes["in"] > 0), sizes
