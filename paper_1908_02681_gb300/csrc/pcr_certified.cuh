@@ -693,13 +693,18 @@ __device__ __forceinline__ PixelEstimate pixel_estimate(const PP& P, float x, fl
   return e;
 }
 
+// w_d <= wf + Delta < near, or w_d >= wf - Delta >= far (directed roundings).
+template <typename PP>
+__device__ __forceinline__ bool certainly_outside_depth(const PP& P, float s, float w) {
+  const float dw = __fmaf_rn(P.kw, s, P.kw3);
+  return (__fadd_ru(w, dw) < P.near_o) | (__fsub_rd(w, dw) >= P.far_o);
+}
+
 // Whether a point that tier 1 did not certify visible is certainly culled.
 template <typename PP>
 __device__ __forceinline__ bool certainly_culled(const PP& P, float s, float w, bool in_range, bool depth_in,
                                                  const PixelEstimate& e) {
-  // By depth: w_d <= wf + Delta < near, or w_d >= wf - Delta >= far (directed roundings).
-  const float dw = __fmaf_rn(P.kw, s, P.kw3);
-  const bool depth_out = (__fadd_ru(w, dw) < P.near_o) | (__fsub_rd(w, dw) >= P.far_o);
+  const bool depth_out = certainly_outside_depth(P, s, w);
   // By the pixel, for a point inside the depth window (wf > 0): b, g from the magnitude sums, and the bound
   // E <= |fm| (9.8u + 1.35 b) + 1.35 g + ce, valid at any |fm| while b <= 1/4.
   const float bf = __fmul_rn(__fmul_rn(__fmaf_rn(P.Mw, s, P.Mw3), e.r), P.cb);

@@ -118,3 +118,12 @@ def test_visible_points_whose_magnitude_sum_overflows(gpu):
     pts = pack(np.column_stack([big, big, -rng.uniform(1.0, 8.0, n)]), rng.integers(0, 1 << 32, n, dtype=np.uint64))
     _, acc = _frames(gpu, _dev(pts), RawView(m, 0.5, 8.5, 64, 48), 0, 1.0, (10, 1))
     assert int((acc[:, 1] >> 32).sum()) == n
+
+
+@pytest.mark.parametrize("looking_away", [False, True])
+def test_clouds_mostly_outside_the_view(gpu, looking_away):
+    """Enough tiles a warp that pass 1 samples the cloud; a camera inside the scan has most points outside its planes."""
+    n = 128 * 152 * 8 * 64 + 12345
+    dev = _dev(scenes.lidar(n, 47))
+    v = scenes.View.lookat((500, 500, 60), (1500, 500, 40) if looking_away else (0, 480, 0), (0, 0, 1), 60.0, 640, 360, 0.1, 300.0)
+    _frames(gpu, dev, v, 0, 1.0, (1, 100), tuning={"blocks_per_sm": 1})
