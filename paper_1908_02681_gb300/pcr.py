@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -145,24 +146,32 @@ def _check(status: int):
         raise PcrError(status, lib.pcr_last_error_message().decode() or lib.pcr_status_string(status).decode())
 
 
+_current = None  # torch's current device and raw stream of a device, once torch's CUDA state exists
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        global _current
+        if _current is None:
+            import torch
+            torch.cuda.current_stream()
+            _current = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+        device, raw = _current
+        return ctypes.c_void_p(raw(device()))
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)
+
+
+_VIEW_HEAD = struct.Struct("=18d")  # view_proj, near_plane, far_plane
 
 
 def make_view(view) -> pcr_view:
     """Marshal a view object (view_proj, near, far and optional depth_mode, metric_scale, ranges,
     transform attributes) into the C struct."""
     v = pcr_view()
-    m = np.ascontiguousarray(np.asarray(view.view_proj, dtype=np.float64).reshape(16))
-    for i in range(16):
-        v.view_proj[i] = float(m[i])
-    v.near_plane = float(view.near)
-    v.far_plane = float(view.far)
+    _VIEW_HEAD.pack_into(v, 0, *np.asarray(view.view_proj, dtype=np.float64).reshape(16).tolist(), float(view.near),
+                         float(view.far))
     v.depth_mode = int(getattr(view, "depth_mode", PCR_DEPTH_LINEAR))
     v.transform = int(getattr(view, "transform", PCR_TRANSFORM_EXACT))
     v.metric_scale = float(getattr(view, "metric_scale", 1000.0))
