@@ -457,7 +457,8 @@ pcr_status pcr_clear(pcr_framebuffer* fb, pcr_stream_t stream) {
   if (pcr_status st = check_fb(fb)) return st;
   fb->band_valid = false;
   const uint64_t npx = (uint64_t)fb->width * fb->height;
-  pcr::k_clear<<<grid_for(npx / 2 + 1, 256, fb->device, 4), 256, 0, (cudaStream_t)stream>>>(fb->keys, fb->accum, npx);
+  pcr::launch_after(pcr::k_clear, grid_for(npx / 2 + 1, 256, fb->device, 4), 256, 0, (cudaStream_t)stream, fb->keys,
+                    fb->accum, npx);
   return after_launch("k_clear");
 }
 
@@ -568,8 +569,8 @@ pcr_status pcr_resolve(pcr_framebuffer* fb, uint32_t* d_rgba_out, uint32_t backg
   if (!(fb->flags & PCR_FB_HQ)) return pcr_resolve_basic(fb, d_rgba_out, background_rgba, clear_after, stream);
   const uint64_t npx = (uint64_t)fb->width * fb->height;
   if (clear_after) fb->band_valid = false;
-  pcr::k_resolve_hq<<<grid_for(npx, 256, fb->device, 4), 256, 0, (cudaStream_t)stream>>>(
-      fb->accum, fb->keys, d_rgba_out, npx, background_rgba, clear_after != 0, fb->status);
+  pcr::launch_after(pcr::k_resolve_hq, grid_for(npx, 256, fb->device, 4), 256, 0, (cudaStream_t)stream, fb->accum, fb->keys,
+                    d_rgba_out, npx, background_rgba, (int)(clear_after != 0), fb->status);
   return after_launch("k_resolve_hq");
 }
 
@@ -579,8 +580,8 @@ pcr_status pcr_resolve_basic(pcr_framebuffer* fb, uint32_t* d_rgba_out, uint32_t
   if (!d_rgba_out) return fail(PCR_ERR_INVALID_ARG, "d_rgba_out is NULL");
   const uint64_t npx = (uint64_t)fb->width * fb->height;
   if (clear_after) fb->band_valid = false;
-  pcr::k_resolve_basic<<<grid_for(npx, 256, fb->device, 4), 256, 0, (cudaStream_t)stream>>>(
-      fb->keys, fb->accum, d_rgba_out, npx, background_rgba, clear_after != 0);
+  pcr::launch_after(pcr::k_resolve_basic, grid_for(npx, 256, fb->device, 4), 256, 0, (cudaStream_t)stream, fb->keys,
+                    fb->accum, d_rgba_out, npx, background_rgba, (int)(clear_after != 0));
   return after_launch("k_resolve_basic");
 }
 
@@ -591,8 +592,8 @@ pcr_status pcr_resolve_both(pcr_framebuffer* fb, uint32_t* d_rgba_basic, uint32_
   if (!d_rgba_basic || !d_rgba_hq) return fail(PCR_ERR_INVALID_ARG, "an output image is NULL");
   const uint64_t npx = (uint64_t)fb->width * fb->height;
   if (clear_after) fb->band_valid = false;
-  pcr::k_resolve_both<<<grid_for(npx, 256, fb->device, 4), 256, 0, (cudaStream_t)stream>>>(
-      fb->keys, fb->accum, d_rgba_basic, d_rgba_hq, npx, background_rgba, clear_after != 0, fb->status);
+  pcr::launch_after(pcr::k_resolve_both, grid_for(npx, 256, fb->device, 4), 256, 0, (cudaStream_t)stream, fb->keys,
+                    fb->accum, d_rgba_basic, d_rgba_hq, npx, background_rgba, (int)(clear_after != 0), fb->status);
   return after_launch("k_resolve_both");
 }
 

@@ -89,6 +89,29 @@ __device__ __forceinline__ bool in_band(unsigned long long q, unsigned long long
   return (unsigned long long)eps_den * (q - qmin) <= (unsigned long long)eps_num * (qmin + nq);
 }
 
+// Programmatic dependent launch. A kernel launched with launch_after may start while the kernel before it on the stream
+// still runs: it does what needs no memory of other kernels (its depth tables), then waits for that kernel's end
+// (wait_previous) before its first access to global memory. release_next lets the next such kernel start early. Kernels
+// of one chain all wait, so the end of one implies the end of those before it; any other kernel, copy or
+// event on the stream is ordered as usual.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, (P)args...);
+}
+
 // Packed HQ increments: {R | G << 32} and {B | 1 << 32}.
 __device__ __forceinline__ unsigned long long hq_rg(uint32_t rgba) {
   return (unsigned long long)(rgba & 0xFFu) | ((unsigned long long)((rgba >> 8) & 0xFFu) << 32);

@@ -8,6 +8,8 @@ namespace pcr {
 // Section 2.1 clear value: keys -> empty; HQ sums and counts -> 0. Two pixels per thread per step
 // (16-byte stores); grid-stride.
 __global__ void k_clear(unsigned long long* __restrict__ keys, ulonglong2* __restrict__ accum, uint64_t npx) {
+  release_next();
+  wait_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t pairs = npx >> 1;
   ulonglong2* k2 = reinterpret_cast<ulonglong2*>(keys);
@@ -87,6 +89,8 @@ __device__ __forceinline__ uint32_t hq_colour(const ulonglong2& a, uint32_t back
 // Section 2.1 resolve: key -> RGBA8; optional clear (keys, and the HQ sums when present).
 __global__ void k_resolve_basic(unsigned long long* __restrict__ keys, ulonglong2* __restrict__ accum,
                                 uint32_t* __restrict__ rgba, uint64_t npx, uint32_t background, int clear) {
+  release_next();
+  wait_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += stride) {
     rgba[i] = basic_colour(keys[i], background);
@@ -101,6 +105,8 @@ __global__ void k_resolve_basic(unsigned long long* __restrict__ keys, ulonglong
 __global__ void k_resolve_hq(ulonglong2* __restrict__ accum, unsigned long long* __restrict__ keys,
                              uint32_t* __restrict__ rgba, uint64_t npx, uint32_t background, int clear,
                              uint32_t* __restrict__ status) {
+  release_next();
+  wait_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   bool overflow = false;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += stride) {
@@ -119,6 +125,8 @@ __global__ void k_resolve_hq(ulonglong2* __restrict__ accum, unsigned long long*
 __global__ void k_resolve_both(unsigned long long* __restrict__ keys, ulonglong2* __restrict__ accum,
                                uint32_t* __restrict__ rgba_basic, uint32_t* __restrict__ rgba_hq, uint64_t npx,
                                uint32_t background, int clear, uint32_t* __restrict__ status) {
+  release_next();
+  wait_previous();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   bool overflow = false;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += stride) {

@@ -358,15 +358,15 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
   const uint32_t lane = threadIdx.x & 31u;
   ScreenQueues& q = reinterpret_cast<ScreenQueues*>(smem + tables * kTableBytes)[threadIdx.x >> 5];
   const WarpTiles T = warp_tiles();
+  release_next();
+  build_tables(P.col, tables, sF);
+  wait_previous();
   bool far_out = false;  // many points outside the clip planes: see kSampleTiles
   if (n / kTile / T.G >= kSampleTiles) {
     const uint4* const sample = pts + (uint64_t)T.g * (n / kTile / T.G) * kTile + lane;
     const uint4 p0 = ld_stream16(sample), p1 = ld_stream16(sample + 32);
-    build_tables(P.col, tables, sF);
     const int out = __syncthreads_count(point_outside_depth(P, p0)) + __syncthreads_count(point_outside_depth(P, p1));
     far_out = 2 * out >= (int)blockDim.x;  // a quarter of the block's 2 blockDim.x sampled points
-  } else {
-    build_tables(P.col, tables, sF);
   }
   uint32_t cn = 0, on = 0;
   auto tier2 = [&](uint32_t place) { raster_deferred(P, sF, point_at(pts, T, place), keys); };
@@ -500,7 +500,9 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
   ScreenQueues& q = reinterpret_cast<ScreenQueues*>(smem + kTableBytes)[warp];
   AddQueue aq{reinterpret_cast<uint2*>(smem + kTableBytes + warps * sizeof(ScreenQueues)) + warp * kAddRing, 0u, 0u};
   const WarpTiles T = warp_tiles();
+  release_next();
   build_tables(P.col, 1, sF);
+  wait_previous();
   uint32_t cn = 0, on = 0;
   auto tier2 = [&](uint32_t place) {
     hq_deferred(P, sF, point_at(pts, T, place), keys, accum, eps_num, eps_den);
@@ -586,7 +588,7 @@ inline void raster_screen_launch(const uint4* pts, uint64_t n, const CertParams&
   static const bool opted = screen_opt_in(k_raster_screen<kMode>, most, false);
   (void)opted;
   const ScreenLaunch L = screen_launch(n, sms, per_sm, table_blocks(P), false);
-  k_raster_screen<kMode><<<L.grid, L.threads, L.smem, s>>>(pts, n, P, S, keys);
+  launch_after(k_raster_screen<kMode>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys);
 }
 
 inline void launch_raster_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
@@ -606,7 +608,7 @@ inline void hq_screen_launch(const uint4* pts, uint64_t n, const CertParams& P, 
   static const bool opted = screen_opt_in(k_hq_screen<kMode>, 1, true);
   (void)opted;
   const ScreenLaunch L = screen_launch(n, sms, per_sm, 1, true);
-  k_hq_screen<kMode><<<L.grid, L.threads, L.smem, s>>>(pts, n, P, S, keys, accum, eps_num, eps_den);
+  launch_after(k_hq_screen<kMode>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, accum, eps_num, eps_den);
 }
 
 inline void launch_hq_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
