@@ -494,18 +494,15 @@ pcr_status pcr_project_points(const pcr_point* d_points, uint64_t n, const pcr_v
   const bool approx = view->transform == PCR_TRANSFORM_DOUBLE_FLOAT;
   if (view->transform == PCR_TRANSFORM_FP64 || !pcr::cached_cert(dv, approx, &P)) {
     pcr::k_project_fp64<<<grid, 256, 0, s>>>(pts, n, dv, d_pixel, keys);
-  } else if (P->n_pw > 0) {
-    const size_t bytes = (size_t)P->n_pw * pcr::kTableBytes;  // PIECEWISE: the ranges' tables
-    auto kernel = P->n_pw > 2 ? pcr::k_project_cert<false, 2> : pcr::k_project_cert<false, 1>;
-    // opt in to the largest size, so that a concurrent call with fewer ranges does not lower the limit
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)(pcr::kMaxRanges * pcr::kTableBytes));
-    if (e != cudaSuccess) return cuda_fail(e, "piecewise projection");
-    kernel<<<grid, 256, bytes, s>>>(pts, n, *P, d_pixel, keys);
-  } else if (approx)
-    pcr::k_project_cert<true><<<grid, 256, 0, s>>>(pts, n, *P, d_pixel, keys);
-  else
-    pcr::k_project_cert<false><<<grid, 256, 0, s>>>(pts, n, *P, d_pixel, keys);
+  } else if (approx) {
+    pcr::k_project_df<<<grid, 256, 0, s>>>(pts, n, *P, d_pixel, keys);
+  } else {
+    const int sms = sm_count(device);
+    const cudaError_t e = P->n_pw > 2   ? pcr::launch_project<2>(pts, n, *P, d_pixel, keys, sms, s)
+                          : P->n_pw > 0 ? pcr::launch_project<1>(pts, n, *P, d_pixel, keys, sms, s)
+                                        : pcr::launch_project<0>(pts, n, *P, d_pixel, keys, sms, s);
+    if (e != cudaSuccess) return cuda_fail(e, "projection");
+  }
   return after_launch("k_project");
 }
 

@@ -127,3 +127,16 @@ def test_clouds_mostly_outside_the_view(gpu, looking_away):
     dev = _dev(scenes.lidar(n, 47))
     v = scenes.View.lookat((500, 500, 60), (1500, 500, 40) if looking_away else (0, 480, 0), (0, 0, 1), 60.0, 640, 360, 0.1, 300.0)
     _frames(gpu, dev, v, 0, 1.0, (1, 100), tuning={"blocks_per_sm": 1})
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 63, 64, 65, 2049, 152 * 256 + 1, 500_003])
+@pytest.mark.parametrize("depth", [0, 1, 2])
+def test_projection_sizes(gpu, n, depth):
+    """pcr_project_points by the exact transform (k_project_cert) against the FP64 kernel, point by point."""
+    import torch
+    dev = _dev(scenes.lidar(n, 48))
+    v = scenes.lidar_1km_view(320, 180)
+    ranges = np.array([[0.0, 10.0, 1e9], [10.0, 600.0, 1e6], [600.0, 5000.0, 1e3]])
+    got = [gpu.pcr_project_points(dev, RawView(np.asarray(v.view_proj), v.near, v.far, 320, 180, depth, 1000.0, ranges, t))
+           for t in (0, 1)]
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
