@@ -321,7 +321,8 @@ pcr_status pcr_batch_set_views(pcr_batch* batch, const pcr_view* views);
  *   - per view, mark the chunks whose bounding box is certainly outside the view (behind the near plane,
  *     beyond the far plane, or at |ndc| > 1 + 1e-5, with margins covering every rounding);
  *   - pass 1 for all views in one persistent launch that skips those chunks and takes the chunk ranges in
- *     turn for every view (so each range is read from HBM once), then pass 2 (hq) likewise. A frame of at
+ *     turn for every view (so each range is read from HBM once), then pass 2 (hq) likewise, or, for clouds of at
+ *     least 2.5 * 10^6 points, one launch per view that skips the view's culled chunks. A frame of at
  *     most 4 views, or of a cloud of at least 10^8 points, instead runs one single-view pass per view,
  *     which is faster there (frames recorded by pcr_batch_capture always use the persistent launch);
  *   - resolve every framebuffer into its output (and clear it, see pcr_batch_create).

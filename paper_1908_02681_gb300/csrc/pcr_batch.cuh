@@ -22,6 +22,7 @@
 namespace pcr {
 
 constexpr int kChunk = 1024;        // points per chunk (bounding box granularity)
+static_assert(kChunk == kTile * (int)kTilesPerChunk, "the screened pass skips whole chunks");
 constexpr int kMaxBatchViews = 256;
 
 // Per-view constants of a batch that live in device memory (read once per work item).

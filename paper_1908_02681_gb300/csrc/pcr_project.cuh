@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_project_cert(const uint4*
       tier2(place);
     }
   };
-  screen_tiles(
+  screen_tiles<false>(
       pts, n, T, lane,
       [&](const uint4& p0, const uint4& p1, uint32_t place) {
         const uint64_t i = index(place);

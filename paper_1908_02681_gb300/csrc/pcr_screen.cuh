@@ -311,30 +311,52 @@ __device__ __forceinline__ uint4 point_at(const uint4* pts, const WarpTiles& T, 
 
 // The full tiles of a warp, both points of a lane at a time, loaded one tile ahead (as stream_direct): body(p0, p1,
 // place of p0); for the partial last tile rest(place of the lane's first point, whether each of its points exists).
-template <typename Body, typename Rest>
+// kMask: the full tiles of chunks whose bit in `mask` is clear (16 tiles a chunk) are skipped; a tile's mask word is read
+// two tiles ahead, so that its points are still requested one ahead.
+constexpr uint32_t kTilesPerChunk = 16;
+
+template <bool kMask, typename Body, typename Rest>
 __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint64_t n, const WarpTiles& T, uint32_t lane,
-                                             Body&& body, Rest&& rest) {
+                                             Body&& body, Rest&& rest, const uint32_t* __restrict__ mask = nullptr) {
   const uint64_t n_full = n / kTile;
   const uint32_t G = T.G, g = T.g;
   const uint32_t tiles = n_full > g ? (uint32_t)((n_full - g - 1u) / G) + 1u : 0u;
   const uint4* p = pts + (uint64_t)g * kTile + lane;
   const uint64_t step = (uint64_t)G * kTile;
   uint4 a0 = make_uint4(0u, 0u, 0u, 0u), a1 = a0;
+  uint32_t chunk = 0, word = 0;  // kMask: the next tile's chunk and its mask word
+  bool seen = true;              // kMask: whether the current tile's chunk is visible
+  auto chunk_of = [&](uint32_t at) { return (uint32_t)((g + (uint64_t)(at >> 6) * G) / kTilesPerChunk); };
+  auto bit = [&](uint32_t w, uint32_t c) { return ((w >> (c & 31u)) & 1u) != 0u; };
   if (tiles) {
-    a0 = ld_stream16(p);
-    a1 = ld_stream16(p + 32);
+    if constexpr (kMask) {
+      const uint32_t c = chunk_of(0);
+      seen = bit(mask[c >> 5], c);
+      chunk = chunk_of(kTile);
+      if (tiles > 1u) word = mask[chunk >> 5];
+    }
+    if (!kMask || seen) {
+      a0 = ld_stream16(p);
+      a1 = ld_stream16(p + 32);
+    }
   }
   const uint32_t end = tiles * (uint32_t)kTile + lane;
   uint32_t place = lane;
 #pragma unroll 1
   while (place != end) {
     const uint4 c0 = a0, c1 = a1;
+    const bool now = seen;
     p += step;
-    if (place + (uint32_t)kTile != end) {
+    if constexpr (kMask) {
+      seen = bit(word, chunk);
+      chunk = chunk_of(place + 2u * kTile);
+      if (end - place > 2u * kTile) word = mask[chunk >> 5];
+    }
+    if (place + (uint32_t)kTile != end && (!kMask || seen)) {
       a0 = ld_stream16(p);
       a1 = ld_stream16(p + 32);
     }
-    body(c0, c1, place);
+    if (!kMask || now) body(c0, c1, place);
     place += (uint32_t)kTile;
   }
   const uint32_t rem = (uint32_t)(n - n_full * kTile);
@@ -402,14 +424,14 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
     drain_batches(q, on, cn, lane, tier2, candidate);
   };
   if (far_out)
-    screen_tiles(
+    screen_tiles<false>(
         pts, n, T, lane,
         [&](const uint4& p0, const uint4& p1, uint32_t place) {
           if (!__all_sync(0xFFFFFFFFu, point_outside_depth(P, p0) & point_outside_depth(P, p1))) tile(p0, p1, place);
         },
         rest);
   else
-    screen_tiles(pts, n, T, lane, tile, rest);
+    screen_tiles<false>(pts, n, T, lane, tile, rest);
   __syncwarp();
   if (cn) candidate(lane < cn ? lane : 0u, lane < cn);
   __syncwarp();
@@ -489,11 +511,12 @@ __device__ __forceinline__ void add_finish(AddQueue& q, unsigned long long* accu
 // (band_bounds_exact): accepted means qmin <= q <= qmin + floor(eps (qmin + Nq)). Same shape and bounds as pass 1. On
 // one GB300, against k_hq_cert: 100M points in scan order 0.680 to 0.46 ms, 37M shuffled 0.290 to 0.22, with the paired
 // additions (see AddQueue) and the screen.
-template <int kMode>
+// kMask: only the chunks whose bit is set in mask (k_cull; a view of a batched frame).
+template <int kMode, bool kMask>
 __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P, const __grid_constant__ Screen S,
     const unsigned long long* __restrict__ keys, unsigned long long* __restrict__ accum, uint32_t eps_num,
-    uint32_t eps_den) {
+    uint32_t eps_den, const uint32_t* __restrict__ mask) {
   extern __shared__ __align__(16) unsigned char smem[];
   long long* const sF = reinterpret_cast<long long*>(smem);
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
@@ -517,7 +540,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
     add_drain_full(aq, accum, lane);
     push_open(valid & !exact, q.place[i], q.open, on, lane);
   };
-  screen_tiles(
+  screen_tiles<kMask>(
       pts, n, T, lane,
       [&](const uint4& p0, const uint4& p1, uint32_t place) {
         const ScreenPoint s0 = screen_point<kMode>(P, S, p0, keys), s1 = screen_point<kMode>(P, S, p1, keys);
@@ -543,7 +566,8 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
         push_open(v0, place, q.open, on, lane);
         push_open(v1, place + 32u, q.open, on, lane);
         drain_batches(q, on, cn, lane, tier2, candidate);
-      });
+      },
+      mask);
   __syncwarp();
   if (cn) candidate(lane < cn ? lane : 0u, lane < cn);
   add_finish(aq, accum, lane);
@@ -601,21 +625,61 @@ inline void launch_raster_screen(const uint4* pts, uint64_t n, const CertParams&
   }
 }
 
-template <int kMode>
-inline void hq_screen_launch(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                             const unsigned long long* keys, unsigned long long* accum, uint32_t eps_num,
-                             uint32_t eps_den, int sms, int per_sm, cudaStream_t s) {
-  static const bool opted = screen_opt_in(k_hq_screen<kMode>, 1, true);
+// One launch of pass 2: the kernel, its shape and its arguments (kept together so that a captured frame's nodes can be
+// given a new view's).
+struct HqScreenLaunch {
+  const uint4* pts;
+  uint64_t n;
+  CertParams P;
+  Screen S;
+  const unsigned long long* keys;
+  unsigned long long* accum;
+  uint32_t eps_num, eps_den;
+  const uint32_t* mask;
+  const void* kernel;
+  ScreenLaunch shape;
+  void* args[9];
+};
+
+template <int kMode, bool kMask>
+inline const void* hq_screen_kernel() {
+  static const bool opted = screen_opt_in(k_hq_screen<kMode, kMask>, 1, true);
   (void)opted;
-  const ScreenLaunch L = screen_launch(n, sms, per_sm, 1, true);
-  launch_after(k_hq_screen<kMode>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, accum, eps_num, eps_den);
+  return reinterpret_cast<const void*>(k_hq_screen<kMode, kMask>);
 }
 
-inline void launch_hq_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                             const unsigned long long* keys, unsigned long long* accum, uint32_t eps_num,
-                             uint32_t eps_den, int sms, int per_sm, cudaStream_t s) {
-  screen_mode(P) == kUnit1 ? hq_screen_launch<kUnit1>(pts, n, P, S, keys, accum, eps_num, eps_den, sms, per_sm, s)
-                           : hq_screen_launch<kUnit256>(pts, n, P, S, keys, accum, eps_num, eps_den, sms, per_sm, s);
+inline void make_hq_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S, const unsigned long long* keys,
+                           unsigned long long* accum, uint32_t eps_num, uint32_t eps_den, const uint32_t* mask, int sms,
+                           int per_sm, HqScreenLaunch* o) {
+  o->pts = pts;
+  o->n = n;
+  o->P = P;
+  o->S = S;
+  o->keys = keys;
+  o->accum = accum;
+  o->eps_num = eps_num;
+  o->eps_den = eps_den;
+  o->mask = mask;
+  const bool unit1 = screen_mode(P) == kUnit1;
+  o->kernel = mask ? (unit1 ? hq_screen_kernel<kUnit1, true>() : hq_screen_kernel<kUnit256, true>())
+                   : (unit1 ? hq_screen_kernel<kUnit1, false>() : hq_screen_kernel<kUnit256, false>());
+  o->shape = screen_launch(n, sms, per_sm, 1, true);
+  void* args[9] = {&o->pts, &o->n, &o->P, &o->S, &o->keys, &o->accum, &o->eps_num, &o->eps_den, &o->mask};
+  std::memcpy(o->args, args, sizeof(args));
+}
+
+inline void launch_hq_screen(HqScreenLaunch& l, cudaStream_t s) {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = l.shape.grid;
+  c.blockDim = l.shape.threads;
+  c.dynamicSmemBytes = l.shape.smem;
+  c.stream = s;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  cudaLaunchKernelExC(&c, l.kernel, l.args);
 }
 
 // Pass 1 of prepared constants with default tuning: screened where the screen applies.
@@ -635,7 +699,11 @@ inline void launch_hq_default(const uint4* pts, uint64_t n, const CertParams& P,
                               int per_sm, bool own_pass1, cudaStream_t s) {
   Screen S;
   if (band_bounds_exact(P.v.nq, eps_num, eps_den) && make_screen(P, eps_num, eps_den, !own_pass1, &S))
-    launch_hq_screen(pts, n, P, S, keys, accum, eps_num, eps_den, sms, per_sm, s);
+  {
+    HqScreenLaunch l;
+    make_hq_screen(pts, n, P, S, keys, accum, eps_num, eps_den, nullptr, sms, per_sm, &l);
+    launch_hq_screen(l, s);
+  }
   else
     hq_launch<false, false>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s);
 }

@@ -27,3 +27,45 @@ def test_items(gpu, n, slice_words):
         for a, b in zip(gpu.pcr_framebuffer_keys(fb), gpu.pcr_framebuffer_keys(one)):
             assert torch.equal(a, b)
     batch.close()
+
+
+def test_captured_views_of_the_screened_pass(gpu):
+    """High-quality frames large enough that pass 2 runs one screened launch per view (with the view's chunk mask): a
+    captured frame follows new views, other depth units, views the screen cannot take (depth codes in units of 1e26 m)
+    and back, and cameras that see little of the cloud, replayed on the legacy default stream."""
+    import torch
+    from tests.helpers import RawView
+    dev = torch.from_numpy(scenes.lidar(2_600_007, 62).view("int32")).cuda()
+    sizes = ((200, 120), (333, 95))
+    fbs, outs = [], []
+    for i in range(6):
+        w, h = sizes[i % 2]
+        fbs.append(gpu.pcr_create_framebuffer(w, h, gpu.PCR_FB_HQ))
+        outs.append(torch.zeros(w * h, dtype=torch.int32, device="cuda"))
+    batch = gpu.pcr_batch_create(gpu.pcr_cloud_create(dev), fbs, outs, True, 1, 100, 0xFF010203, True)
+
+    def views(seed, depth, scale, near_ground=False):
+        vs = scenes.orbit_views(6, seed, resolutions=sizes)
+        if near_ground:
+            vs = [scenes.View.lookat((300 + 90 * i, 500, 60), (300 + 90 * i, 560, 20), (0, 0, 1), 60.0, *sizes[i % 2], 0.1, 120.0)
+                  for i in range(6)]
+        return [RawView(v.view_proj, v.near, v.far, v.width, v.height, depth, scale) for v in vs]
+
+    first = True
+    for vs in (views(3, 0, 1.0), views(4, 0, 1.0), views(5, 1, 1000.0), views(6, 1, 1e-26), views(7, 0, 1.0, True),
+               views(8, 1, 1e8)):
+        gpu.pcr_batch_set_views(batch, vs)
+        if first:
+            gpu.pcr_batch_capture(batch, torch.cuda.Stream())
+            first = False
+        for o in outs:
+            o.zero_()
+        gpu.pcr_batch_launch(batch, 0)
+        torch.cuda.synchronize()
+        for v, o in zip(vs, outs):
+            one = gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ)
+            want = torch.empty_like(o)
+            gpu.pcr_render_hq_splat(one, dev, v, 1, 100)
+            gpu.pcr_resolve(one, want, 0xFF010203, clear_after=True)
+            assert torch.equal(o, want)
+    batch.close()
