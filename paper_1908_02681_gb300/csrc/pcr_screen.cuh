@@ -126,8 +126,9 @@ struct ScreenPoint {
   bool open;   // undecided, and not certainly culled (tier 2 decides)
 };
 
-// Both points of a lane, as pass 1 takes them, with one cull branch for the two. (Pass 2 keeps screen_point: with one
-// cull branch its 37M shuffled points took 3 % longer.)
+// Both points of a lane. One branch leads to the cull tests of the two: on scans a tile mostly has none of them (pass 2 of
+// the 100M-point scan on one GB300 1.5 % faster than with a branch per point, 400M city points' pass 1 5 %; 37M shuffled
+// points' pass 2 1 % slower).
 struct ScreenTwo {
   ScreenPoint a, b;
 };
@@ -163,9 +164,10 @@ __device__ __forceinline__ ScreenTwo screen_two(const CertParams& P, const Scree
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       ScreenPoint& o = h ? t.b : t.a;
-      const bool out = certainly_culled(P, s[h], o.w, s[h] < P.xyz_max, in[h], e[h]);
-      o.w = o.open ? __int_as_float(0x7F800000) : o.w;
-      o.open &= !out;
+      if (o.open) {
+        o.open = !certainly_culled(P, s[h], o.w, s[h] < P.xyz_max, in[h], e[h]);
+        o.w = __int_as_float(0x7F800000);
+      }
     }
   }
   return t;
@@ -179,45 +181,21 @@ __device__ __forceinline__ bool point_outside_depth(const CertParams& P, const u
   return (s < P.xyz_max) & certainly_outside_depth(P, s, w);
 }
 
-template <int kMode>
-__device__ __forceinline__ ScreenPoint screen_point(const CertParams& P, const Screen& S, const uint4& p,
-                                                    const unsigned long long* keys) {
-  const float x = __uint_as_float(p.x), y = __uint_as_float(p.y), z = __uint_as_float(p.z);
-  const float s = __fadd_rn(__fadd_rn(fabsf(x), fabsf(y)), fabsf(z));
-  ScreenPoint o;
-  o.w = __fmaf_rn(P.Wr[2], z, __fmaf_rn(P.Wr[1], y, __fmaf_rn(P.Wr[0], x, P.Wr[3])));
-  const int r = screen_range<kMode>(P, o.w);
-  constexpr bool kPw = kMode >= kPiecewise2;
-  const float wc = kPw ? ranged<kMode>(P.pw_wc, r) : P.wc, whk = kPw ? ranged<kMode>(P.pw_whk, r) : P.whk;
-  const bool depth_in = fabsf(__fsub_rn(o.w, wc)) < __fmaf_rn(-P.kw, s, whk);
-  const PixelEstimate e = pixel_estimate(P, x, y, z, s, o.w);
-  o.m = __fmaf_rn(S.k, s, ranged<kMode>(S.k3, r));
-  o.a = ranged<kMode>(S.a, r);
-  o.b = ranged<kMode>(S.b, r);
-  o.pixel = e.pixel;
-  o.k = 0.0f;
-  o.open = false;
-  if (depth_in & e.ok) {
-    o.k = stored_depth<kMode>(keys, o.pixel);
-  } else {
-    o.open = !certainly_culled(P, s, o.w, s < P.xyz_max, depth_in, e);
-    o.w = __int_as_float(0x7F800000);
-  }
-  return o;
-}
-
 // Per-warp queues in shared memory: two pushes of 32 on top of at most 31 left over. Points are also known by their
 // place in the warp's sequence of tiles: 64 * tile number + place in the tile (fits 32 bits: n < 2^40, and a grid over
 // that many points has over 1000 warps). Open points are queued by place alone and read again for tier 2: they are
-// few, and shared memory that the queues leave free is L1, which holds the stored-key reads in flight (reading the
-// candidates again as well cost more than their space: the 100M-point frame 1.13 against 1.06 ms).
+// few, and shared memory that the queues leave free is L1, which holds the stored-key reads in flight. Pass 1 keeps its
+// candidates' points (reading them again cost more than their space: the 100M-point frame 1.13 against 1.06 ms), pass 2,
+// with few candidates, does not (that frame 0.97 to 0.95 ms on one GB300; 37M shuffled points 0.442 to 0.452).
 constexpr uint32_t kCand = 96;
 
-struct ScreenQueues {
-  uint4 p[kCand];         // candidates: certainly visible points whose exact code decides,
-  uint32_t pixel[kCand];  // their pixels
+struct PlaceQueues {
+  uint32_t pixel[kCand];  // candidates: certainly visible points whose exact code decides, their pixels
   uint32_t place[kCand];  // and places
   uint32_t open[kCand];   // places of the points for tier 2
+};
+struct ScreenQueues : PlaceQueues {  // pass 1, whose candidates are many
+  uint4 p[kCand];
 };
 
 // Threads of a screened pass's block at most: one block an SM (see k_raster_screen); launches over few points take
@@ -272,11 +250,23 @@ __device__ __forceinline__ void push_candidate(bool need, const uint4& p, uint32
   qn += __popc(m);
 }
 
+// The same for pass 2, whose candidates (next to a band edge) are few and read again.
+__device__ __forceinline__ void push_candidate(bool need, uint32_t pixel, uint32_t place, PlaceQueues& q, uint32_t& qn,
+                                               uint32_t lane) {
+  const unsigned m = __ballot_sync(0xFFFFFFFFu, need);
+  if (need) {
+    const uint32_t i = qn + __popc(m & ((1u << lane) - 1u));
+    q.pixel[i] = pixel;
+    q.place[i] = place;
+  }
+  qn += __popc(m);
+}
+
 // Runs tier2(place) and candidate(index, true) on batches of 32 while there are that many. Called at the end of a
 // tile, where few registers are live across the out-of-line tier 2. A candidate batch leaves at most 32 open points,
 // which go first. All lanes must call it.
 template <typename T2, typename Cand>
-__device__ __forceinline__ void drain_batches(ScreenQueues& q, uint32_t& on, uint32_t& cn, uint32_t lane, T2&& tier2,
+__device__ __forceinline__ void drain_batches(PlaceQueues& q, uint32_t& on, uint32_t& cn, uint32_t lane, T2&& tier2,
                                               Cand&& candidate) {
   __syncwarp();
   for (;;) {
@@ -459,26 +449,18 @@ __device__ __forceinline__ void add_drain(const AddQueue& q, unsigned long long*
   const uint4 e0 = e[0], e1 = e[1];  // entries 4g .. 4g + 3: {pixel, rgba, pixel, rgba}
   // the lane's word of each entry as two 16-bit halves: {R, G}, or {B, 1}; four of them cannot carry
   const uint32_t sel = lane & 1u ? 0x5452u : 0x5150u;
-  uint32_t pix = e0.x, sum = __byte_perm(e0.y, 1u, sel);
   unsigned long long* const acc = accum + (lane & 1u);
-  auto flush = [&]() {
-    if (!kGuard || pix != 0xFFFFFFFFu)
+  const bool same1 = e0.z == e0.x, same2 = e1.x == e0.z, same3 = e1.z == e1.x;  // as the entry before
+  const uint32_t s3 = __byte_perm(e1.w, 1u, sel), s2 = __byte_perm(e1.y, 1u, sel) + (same3 ? s3 : 0u),
+                 s1 = __byte_perm(e0.w, 1u, sel) + (same2 ? s2 : 0u), s0 = __byte_perm(e0.y, 1u, sel) + (same1 ? s1 : 0u);
+  auto put = [&](bool first, uint32_t pix, uint32_t sum) {  // the first entry of each run adds the run's sum
+    if (first && (!kGuard || pix != 0xFFFFFFFFu))
       atomicAdd(acc + 2 * (uint64_t)pix, (unsigned long long)(sum & 0xFFFFu) | ((unsigned long long)(sum >> 16) << 32));
   };
-  auto next = [&](uint32_t p, uint32_t rgba) {
-    const uint32_t v = __byte_perm(rgba, 1u, sel);
-    if (p != pix) {
-      flush();
-      pix = p;
-      sum = v;
-    } else {
-      sum += v;
-    }
-  };
-  next(e0.z, e0.w);
-  next(e1.x, e1.y);
-  next(e1.z, e1.w);
-  flush();
+  put(true, e0.x, s0);
+  put(!same1, e0.z, s1);
+  put(!same2, e1.x, s2);
+  put(!same3, e1.z, s3);
 }
 
 // Queues the accepting lanes' fragments. At most two pushes between drains (63 + 64 entries fit the ring).
@@ -509,7 +491,7 @@ __device__ __forceinline__ void add_finish(AddQueue& q, unsigned long long* accu
 
 // Pass 2 (Section 2.2), exact transform, LINEAR or METRIC depth, for bands whose u64 test does not wrap
 // (band_bounds_exact): accepted means qmin <= q <= qmin + floor(eps (qmin + Nq)). Same shape and bounds as pass 1. On
-// one GB300, against k_hq_cert: 100M points in scan order 0.680 to 0.46 ms, 37M shuffled 0.290 to 0.22, with the paired
+// one GB300, against k_hq_cert: 100M points in scan order 0.680 to 0.44 ms, 37M shuffled 0.290 to 0.23, with the paired
 // additions (see AddQueue) and the screen.
 // kMask: only the chunks whose bit is set in mask (k_cull; a view of a batched frame).
 template <int kMode, bool kMask>
@@ -520,8 +502,8 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
   extern __shared__ __align__(16) unsigned char smem[];
   long long* const sF = reinterpret_cast<long long*>(smem);
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  ScreenQueues& q = reinterpret_cast<ScreenQueues*>(smem + kTableBytes)[warp];
-  AddQueue aq{reinterpret_cast<uint2*>(smem + kTableBytes + warps * sizeof(ScreenQueues)) + warp * kAddRing, 0u, 0u};
+  AddQueue aq{reinterpret_cast<uint2*>(smem + kTableBytes) + warp * kAddRing, 0u, 0u};
+  PlaceQueues& q = reinterpret_cast<PlaceQueues*>(smem + kTableBytes + warps * kAddRing * sizeof(uint2))[warp];
   const WarpTiles T = warp_tiles();
   release_next();
   build_tables(P.col, 1, sF);
@@ -531,7 +513,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
     hq_deferred(P, sF, point_at(pts, T, place), keys, accum, eps_num, eps_den);
   };
   auto candidate = [&](uint32_t i, bool valid) {
-    const uint4 p = q.p[i];
+    const uint4 p = point_at(pts, T, q.place[i]);
     const uint32_t pixel = q.pixel[i];
     const unsigned long long qmin = stored_key(keys, pixel) >> 24;
     FixedCode f;
@@ -543,7 +525,8 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
   screen_tiles<kMask>(
       pts, n, T, lane,
       [&](const uint4& p0, const uint4& p1, uint32_t place) {
-        const ScreenPoint s0 = screen_point<kMode>(P, S, p0, keys), s1 = screen_point<kMode>(P, S, p1, keys);
+        const ScreenTwo two = screen_two<kMode>(P, S, p0, p1, keys);
+        const ScreenPoint &s0 = two.a, &s1 = two.b;
         if (__any_sync(0xFFFFFFFFu, s0.open | s1.open)) {
           push_open(s0.open, place, q.open, on, lane);
           push_open(s1.open, place + 32u, q.open, on, lane);
@@ -557,8 +540,8 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
         add_drain_full(aq, accum, lane);
         const bool n0 = fabsf(d0) < s0.m, n1 = fabsf(d1) < s1.m;
         if (__any_sync(0xFFFFFFFFu, n0 | n1)) {
-          push_candidate(n0, p0, s0.pixel, place, q, cn, lane);
-          push_candidate(n1, p1, s1.pixel, place + 32u, q, cn, lane);
+          push_candidate(n0, s0.pixel, place, q, cn, lane);
+          push_candidate(n1, s1.pixel, place + 32u, q, cn, lane);
         }
         if ((on | cn) >= 32u) drain_batches(q, on, cn, lane, tier2, candidate);
       },
@@ -586,7 +569,7 @@ struct ScreenLaunch {
 };
 
 constexpr size_t screen_smem(int warps, int tables, bool hq) {
-  return tables * kTableBytes + (size_t)warps * (sizeof(ScreenQueues) + (hq ? kAddRing * sizeof(uint2) : 0));
+  return tables * kTableBytes + (size_t)warps * (hq ? sizeof(PlaceQueues) + kAddRing * sizeof(uint2) : sizeof(ScreenQueues));
 }
 
 inline ScreenLaunch screen_launch(uint64_t n, int sms, int per_sm, int tables, bool hq) {
