@@ -256,6 +256,22 @@ ulonglong2* bounds_buffer(pcr_framebuffer* fb, cudaStream_t s) {
   return fb->bounds;
 }
 
+// A frame whose two passes run here with default tuning (fb's band mask holds pass 1's words for pass 2, see
+// k_raster_screen): the screen of both, or false (then the passes run without). Not under capture: the buffer may grow, and
+// a replay would write the old one.
+bool frame_words(pcr_framebuffer* fb, uint64_t n, const pcr::DevView& dv, int transform, uint32_t eps_num, uint32_t eps_den,
+                 cudaStream_t s, const pcr::CertParams** P, pcr::Screen* S) {
+  const pcr::Tuning& t = fb->tuning;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  return transform == PCR_TRANSFORM_EXACT && !t.merge && !t.staging && !t.band_filter &&
+         !t.band_bounds && pcr::cached_cert(dv, false, P) && pcr::frame_screen(**P, n, sm_count(fb->device), t.blocks_per_sm, eps_num, eps_den, S) &&
+         band_reserve(fb, n, s);
+}
+
 pcr_status launch_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr::DevView& dv,
                      int transform, uint32_t eps_num, uint32_t eps_den, cudaStream_t s, bool own_pass1) {
   const uint4* pts = reinterpret_cast<const uint4*>(d_points);
@@ -273,6 +289,27 @@ pcr_status launch_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n,
                                                 band ? fb->band_mask : nullptr,
                                                 fb->tuning.band_bounds ? bounds_buffer(fb, s) : nullptr, own_pass1);
   return after_launch("k_hq_certified", (uint64_t)launched);
+}
+
+// Both passes of a high-quality frame.
+pcr_status render_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr::DevView& dv, int transform,
+                     uint32_t eps_num, uint32_t eps_den, cudaStream_t s) {
+  const pcr::CertParams* P = nullptr;
+  pcr::Screen S;
+  if (frame_words(fb, n, dv, transform, eps_num, eps_den, s, &P, &S)) {
+    const uint4* pts = reinterpret_cast<const uint4*>(d_points);
+    const int sms = sm_count(fb->device), per_sm = fb->tuning.blocks_per_sm;
+    pcr::launch_raster_screen(pts, n, *P, S, fb->keys, reinterpret_cast<uint2*>(fb->band_mask), sms, per_sm, s);
+    pcr::HqScreenLaunch l;
+    pcr::make_hq_screen(pts, n, *P, S, fb->keys, reinterpret_cast<unsigned long long*>(fb->accum), eps_num, eps_den,
+                        pcr::kBandWords, fb->band_mask, sms, per_sm, &l);
+    pcr::launch_hq_screen(l, s);
+    return after_launch("screened frame", 2);
+  }
+  const pcr_status st = fb->tuning.band_filter ? launch_raster_band(fb, d_points, n, dv, transform, eps_num, eps_den, s)
+                                               : launch_raster(fb, d_points, n, dv, transform, s);
+  if (st != PCR_OK) return st;
+  return launch_hq(fb, d_points, n, dv, transform, eps_num, eps_den, s, true);
 }
 
 }  // namespace
@@ -410,9 +447,8 @@ pcr_status pcr_autotune(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t
     for (int rep = 0; rep < 2 && st == PCR_OK; ++rep) {
       if ((st = pcr_clear(fb, stream)) != PCR_OK) break;
       cudaEventRecord(e0, s);
-      st = hq && fb->tuning.band_filter ? launch_raster_band(fb, d_points, n, dv, view->transform, 1, 100, s)
-                                        : launch_raster(fb, d_points, n, dv, view->transform, s);
-      if (st == PCR_OK && hq) st = launch_hq(fb, d_points, n, dv, view->transform, 1, 100, s, true);
+      st = hq ? render_hq(fb, d_points, n, dv, view->transform, 1, 100, s)
+              : launch_raster(fb, d_points, n, dv, view->transform, s);
       cudaEventRecord(e1, s);
       if (cudaEventSynchronize(e1) != cudaSuccess) st = cuda_fail(cudaGetLastError(), "autotune timing");
       float ms = 0.f;
@@ -544,11 +580,7 @@ pcr_status pcr_render_hq_splat(pcr_framebuffer* fb, const pcr_point* d_points, u
   if (pcr_status st = check_hq(fb, d_points, n, view, eps_num, eps_den, &dv)) return st;
   if (n == 0) return PCR_OK;
   const cudaStream_t s = (cudaStream_t)stream;
-  const pcr_status st = fb->tuning.band_filter ? launch_raster_band(fb, d_points, n, dv, view->transform, eps_num,
-                                                                    eps_den, s)
-                                               : launch_raster(fb, d_points, n, dv, view->transform, s);
-  if (st != PCR_OK) return st;
-  return launch_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, s, true);
+  return render_hq(fb, d_points, n, dv, view->transform, eps_num, eps_den, s);
 }
 
 pcr_status pcr_hq_accumulate(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr_view* view,

@@ -207,12 +207,6 @@ constexpr int kScreenThreads = 1024;
 // or 40 points: within 1 %) against 0.58 with every candidate queued.
 constexpr int kDirect = 24;
 
-// Pass 1 over at least this many tiles a warp samples the cloud first, a tile a warp spread over all of it: where a
-// quarter of a block's sampled points lie outside the clip planes (scans much larger than the view), it tests each tile
-// for lying outside as a whole before the pixel work. 400M city points on one GB300: 1.32 to 1.11 ms; done always, the
-// test costs the 100M-point scan 2 % of pass 1 and piecewise depth 6 %. The sample costs about a microsecond.
-constexpr uint32_t kSampleTiles = 128;
-
 // Exact code of a certainly visible point (tier 1's depth part; PIECEWISE: with its range's table and constants);
 // false when undecided between two neighbours.
 template <int kMode>
@@ -318,12 +312,17 @@ __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint
   bool seen = true;              // kMask: whether the current tile's chunk is visible
   auto chunk_of = [&](uint32_t at) { return (uint32_t)((g + (uint64_t)(at >> 6) * G) / kTilesPerChunk); };
   auto bit = [&](uint32_t w, uint32_t c) { return ((w >> (c & 31u)) & 1u) != 0u; };
+  auto mask_word = [&](uint32_t c) {  // volatile: not moved above the wait for the kernel that wrote it
+    uint32_t w;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(w) : "l"(mask + (c >> 5)) : "memory");
+    return w;
+  };
   if (tiles) {
     if constexpr (kMask) {
       const uint32_t c = chunk_of(0);
-      seen = bit(mask[c >> 5], c);
+      seen = bit(mask_word(c), c);
       chunk = chunk_of(kTile);
-      if (tiles > 1u) word = mask[chunk >> 5];
+      if (tiles > 1u) word = mask_word(chunk);
     }
     if (!kMask || seen) {
       a0 = ld_stream16(p);
@@ -340,7 +339,7 @@ __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint
     if constexpr (kMask) {
       seen = bit(word, chunk);
       chunk = chunk_of(place + 2u * kTile);
-      if (end - place > 2u * kTile) word = mask[chunk >> 5];
+      if (end - place > 2u * kTile) word = mask_word(chunk);
     }
     if (place + (uint32_t)kTile != end && (!kMask || seen)) {
       a0 = ld_stream16(p);
@@ -353,6 +352,114 @@ __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint
   if (rem != 0u && n_full % G == g) rest(end, lane < rem, lane + 32u < rem);
 }
 
+// A pass over at least this many tiles a warp samples the cloud first, a tile a warp spread over all of it (1.5 us, 1 % of
+// a frame of 25M points, hence the line), and its blocks take the loop that suits it:
+//   far_out: a quarter of the sampled points lie outside the clip planes (scans much larger than the view): pass 1 tests
+//     each tile for lying outside as a whole before the pixel work. 400M city points on one GB300: 1.32 to 1.11 ms; done
+//     always, the test costs the 100M-point scan 2 % of pass 1 and piecewise depth 6 %.
+//   random: fewer than one in 64 of the sampled visible points share their pixel with the next point (clouds in no
+//     order): in HQ frames, pass 1 leaves pass 2 words that say which points it may accept (kBand). Pixels meet their
+//     nearest points early then, and pass 2 reads 38 % of 37M shuffled points: the frame 0.44 to 0.38 ms on one GB300. In scan order
+//     the words leave 60 to 80 % of the points and cost more than they save (100M points 0.94 to 1.00 ms).
+// A block's decision depends on the cloud, the view and the launch shape alone: pass 2, of the same shape, comes to the
+// same one for the same tiles.
+constexpr uint32_t kSampleTiles = 96;
+
+struct CloudSample {
+  bool far_out, random;
+};
+
+template <int kMode>
+__device__ __forceinline__ CloudSample sample_cloud(const CertParams& P, const uint4* pts, uint64_t n, const WarpTiles& T,
+                                                    uint32_t lane) {
+  CloudSample c{false, false};
+  const uint64_t spread = n / kTile / T.G;
+  if (spread < kSampleTiles) return c;
+  // the block's samples lie all over the cloud
+  const uint4* const at = pts + ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * spread * kTile + lane;
+  const uint4 p[2] = {ld_stream16(at), ld_stream16(at + 32)};
+  int outside = 0, seen = 0, same = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float x = __uint_as_float(p[h].x), y = __uint_as_float(p[h].y), z = __uint_as_float(p[h].z);
+    const float s = __fadd_rn(__fadd_rn(fabsf(x), fabsf(y)), fabsf(z));
+    const float w = __fmaf_rn(P.Wr[2], z, __fmaf_rn(P.Wr[1], y, __fmaf_rn(P.Wr[0], x, P.Wr[3])));
+    const PixelEstimate e = pixel_estimate(P, x, y, z, s, w);
+    const uint32_t pixel = w > 0.0f && e.ok ? e.pixel : 0xFFFFFFFFu - lane;
+    outside += __syncthreads_count(point_outside_depth(P, p[h]));
+    seen += __syncthreads_count(w > 0.0f && e.ok);
+    same += __syncthreads_count(__shfl_down_sync(0xFFFFFFFFu, pixel, 1) == pixel && lane < 31u);
+  }
+  c.far_out = 2 * outside >= (int)blockDim.x;
+  c.random = 64 * same < seen;
+  return c;
+}
+
+// The points whose bit is set in `words` (two words a tile of 64), 64 at a time: body(p0, p1, their places, whether each
+// exists). Places are gathered in the warp's queue from the words alone, so tiles without a set bit are not read; a
+// batch's points are requested while the batch before it is processed. The words are read 32 tiles at a time, one ahead.
+constexpr uint32_t kBandQueue = 128;  // at most 63 left over and 64 of a tile
+
+// volatile: not moved above the wait for the kernel that wrote the words
+__device__ __forceinline__ uint2 ld_words(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.global.cs.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  return v;
+}
+
+template <typename Body>
+__device__ __forceinline__ void band_points(const uint4* __restrict__ pts, uint64_t n, const WarpTiles& T, uint32_t lane,
+                                            const uint2* __restrict__ words, uint32_t* q, Body&& body) {
+  const uint64_t n_tiles = (n + kTile - 1) / kTile;
+  const uint32_t tiles = n_tiles > T.g ? (uint32_t)((n_tiles - T.g - 1u) / T.G) + 1u : 0u;
+  auto block = [&](uint32_t t) {  // the words of tiles t + lane
+    return t + lane < tiles ? ld_words(words + T.g + (uint64_t)(t + lane) * T.G) : make_uint2(0u, 0u);
+  };
+  uint2 w = make_uint2(0u, 0u), ahead = block(0);
+  uint32_t t = 0, cn = 0;
+  auto fill = [&]() {
+    while (cn < 64u && t < tiles) {
+      if ((t & 31u) == 0u) {
+        w = ahead;
+        ahead = block(t + 32u);
+      }
+      const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, w.x, t & 31u), b1 = __shfl_sync(0xFFFFFFFFu, w.y, t & 31u);
+      const uint32_t below = (1u << lane) - 1u, place = t * (uint32_t)kTile + lane;
+      if ((b0 >> lane) & 1u) q[cn + __popc(b0 & below)] = place;
+      cn += __popc(b0);
+      if ((b1 >> lane) & 1u) q[cn + __popc(b1 & below)] = place + 32u;
+      cn += __popc(b1);
+      ++t;
+    }
+    __syncwarp();
+  };
+  uint4 a0 = make_uint4(0u, 0u, 0u, 0u), a1 = a0;
+  uint32_t l0 = 0, l1 = 0, have = 0;  // the next batch: places and size
+  auto take = [&]() {
+    fill();
+    have = cn < 64u ? cn : 64u;
+    cn -= have;
+    if (lane < have) {
+      l0 = q[cn + lane];
+      a0 = point_at(pts, T, l0);
+    }
+    if (lane + 32u < have) {
+      l1 = q[cn + lane + 32u];
+      a1 = point_at(pts, T, l1);
+    }
+    __syncwarp();
+  };
+  take();
+#pragma unroll 1
+  while (have) {
+    const uint4 p0 = a0, p1 = a1;
+    const uint32_t c0 = l0, c1 = l1;
+    const bool v0 = lane < have, v1 = lane + 32u < have;
+    take();
+    body(p0, p1, c0, c1, v0, v1);
+  }
+}
+
 // Pass 1 (Section 2.1), exact transform. Issue slots and the latency of the stored-key reads
 // bound it (61 % busy and the top stall at 20M points). 32 warps an SM at 64 registers, as one block: 48 warps with one
 // point a lane (40 registers) and 24 warps (80) were slower, and one block holds one table, which leaves L1 more room
@@ -360,10 +467,12 @@ __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint
 // k_raster_cert, which computes every point's code, on one GB300: 400M city points at 4K 2.23 to 1.41 ms (the culled
 // points), 37M shuffled 0.227 to 0.18, 100M in scan order 0.539 to 0.51, and frames of 0.5 to 4 points per pixel equal
 // or a few per cent faster, so it runs at every size.
-template <int kMode>
+// kBand (HQ frames): also writes, per tile, a bit for each point that pass 2 may accept: clear where the point is culled or
+// certainly beyond the upper band edge of the key its pixel holds (a stored key only decreases, and the edge with it).
+template <int kMode, bool kBand>
 __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P, const __grid_constant__ Screen S,
-    unsigned long long* __restrict__ keys) {
+    unsigned long long* __restrict__ keys, uint2* __restrict__ band) {
   extern __shared__ __align__(16) unsigned char smem[];
   long long* const sF = reinterpret_cast<long long*>(smem);
   const int tables = kMode >= kPiecewise2 ? P.n_pw : 1;
@@ -373,13 +482,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
   release_next();
   build_tables(P.col, tables, sF);
   wait_previous();
-  bool far_out = false;  // many points outside the clip planes: see kSampleTiles
-  if (n / kTile / T.G >= kSampleTiles) {
-    const uint4* const sample = pts + (uint64_t)T.g * (n / kTile / T.G) * kTile + lane;
-    const uint4 p0 = ld_stream16(sample), p1 = ld_stream16(sample + 32);
-    const int out = __syncthreads_count(point_outside_depth(P, p0)) + __syncthreads_count(point_outside_depth(P, p1));
-    far_out = 2 * out >= (int)blockDim.x;  // a quarter of the block's 2 blockDim.x sampled points
-  }
+  const CloudSample sample = sample_cloud<kMode>(P, pts, n, T, lane);
   uint32_t cn = 0, on = 0;
   auto tier2 = [&](uint32_t place) { raster_deferred(P, sF, point_at(pts, T, place), keys); };
   auto commit = [&](bool need, const uint4& p, uint32_t pixel, uint32_t place) {
@@ -389,9 +492,16 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
     if (__any_sync(0xFFFFFFFFu, need & !exact)) push_open(need & !exact, place, q.open, on, lane);
   };
   auto candidate = [&](uint32_t i, bool valid) { commit(valid, q.p[i], q.pixel[i], q.place[i]); };
-  auto tile = [&](const uint4& p0, const uint4& p1, uint32_t place) {
+  auto record = [&](bool b0, bool b1, uint32_t place) {
+    const unsigned m0 = __ballot_sync(0xFFFFFFFFu, b0), m1 = __ballot_sync(0xFFFFFFFFu, b1);
+    if (lane == 0) band[T.g + (uint64_t)(place >> 6) * T.G] = make_uint2(m0, m1);
+  };
+  auto tile = [&](const uint4& p0, const uint4& p1, uint32_t place, bool words) {
         const ScreenTwo two = screen_two<kMode>(P, S, p0, p1, keys);
         const ScreenPoint &s0 = two.a, &s1 = two.b;
+        if (words)
+          record(s0.open | (__fsub_rn(__fmaf_rn(s0.k, S.hi_a, S.hi_b), s0.w) > -s0.m),
+                 s1.open | (__fsub_rn(__fmaf_rn(s1.k, S.hi_a, S.hi_b), s1.w) > -s1.m), place);
         if (__any_sync(0xFFFFFFFFu, s0.open | s1.open)) {
           push_open(s0.open, place, q.open, on, lane);
           push_open(s1.open, place + 32u, q.open, on, lane);
@@ -409,19 +519,24 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
         if ((on | cn) >= 32u) drain_batches(q, on, cn, lane, tier2, candidate);
       };
   auto rest = [&](uint32_t place, bool v0, bool v1) {
+    if (kBand && sample.random) record(v0, v1, place);
     push_open(v0, place, q.open, on, lane);
     push_open(v1, place + 32u, q.open, on, lane);
     drain_batches(q, on, cn, lane, tier2, candidate);
   };
-  if (far_out)
+  auto plain = [&](const uint4& p0, const uint4& p1, uint32_t place) { tile(p0, p1, place, false); };
+  if (kBand && sample.random)
+    screen_tiles<false>(
+        pts, n, T, lane, [&](const uint4& p0, const uint4& p1, uint32_t place) { tile(p0, p1, place, true); }, rest);
+  else if (sample.far_out)
     screen_tiles<false>(
         pts, n, T, lane,
         [&](const uint4& p0, const uint4& p1, uint32_t place) {
-          if (!__all_sync(0xFFFFFFFFu, point_outside_depth(P, p0) & point_outside_depth(P, p1))) tile(p0, p1, place);
+          if (!__all_sync(0xFFFFFFFFu, point_outside_depth(P, p0) & point_outside_depth(P, p1))) plain(p0, p1, place);
         },
         rest);
   else
-    screen_tiles<false>(pts, n, T, lane, tile, rest);
+    screen_tiles<false>(pts, n, T, lane, plain, rest);
   __syncwarp();
   if (cn) candidate(lane < cn ? lane : 0u, lane < cn);
   __syncwarp();
@@ -493,8 +608,11 @@ __device__ __forceinline__ void add_finish(AddQueue& q, unsigned long long* accu
 // (band_bounds_exact): accepted means qmin <= q <= qmin + floor(eps (qmin + Nq)). Same shape and bounds as pass 1. On
 // one GB300, against k_hq_cert: 100M points in scan order 0.680 to 0.44 ms, 37M shuffled 0.290 to 0.23, with the paired
 // additions (see AddQueue) and the screen.
-// kMask: only the chunks whose bit is set in mask (k_cull; a view of a batched frame).
-template <int kMode, bool kMask>
+// kFrom: every tile; the tiles of the chunks whose bit is set in `mask` (k_cull; a view of a batched frame); or the points
+// whose bit is set in the words that pass 1 wrote (`mask`, two words a tile; see k_raster_screen).
+enum HqSource : int { kAllTiles = 0, kChunkMask = 1, kBandWords = 2 };
+
+template <int kMode, int kFrom>
 __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P, const __grid_constant__ Screen S,
     const unsigned long long* __restrict__ keys, unsigned long long* __restrict__ accum, uint32_t eps_num,
@@ -522,35 +640,50 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_hq_screen(
     add_drain_full(aq, accum, lane);
     push_open(valid & !exact, q.place[i], q.open, on, lane);
   };
-  screen_tiles<kMask>(
-      pts, n, T, lane,
-      [&](const uint4& p0, const uint4& p1, uint32_t place) {
-        const ScreenTwo two = screen_two<kMode>(P, S, p0, p1, keys);
-        const ScreenPoint &s0 = two.a, &s1 = two.b;
-        if (__any_sync(0xFFFFFFFFu, s0.open | s1.open)) {
-          push_open(s0.open, place, q.open, on, lane);
-          push_open(s1.open, place + 32u, q.open, on, lane);
-        }
-        auto inside = [&](const ScreenPoint& o) {  // >= m: in the band; <= -m: outside it
-          return fminf(__fsub_rn(o.w, __fmaf_rn(o.k, S.lo_a, S.lo_b)), __fsub_rn(__fmaf_rn(o.k, S.hi_a, S.hi_b), o.w));
-        };
-        const float d0 = inside(s0), d1 = inside(s1);
-        add_push(d0 >= s0.m, s0.pixel, p0.w, aq, lane);
-        add_push(d1 >= s1.m, s1.pixel, p1.w, aq, lane);
-        add_drain_full(aq, accum, lane);
-        const bool n0 = fabsf(d0) < s0.m, n1 = fabsf(d1) < s1.m;
-        if (__any_sync(0xFFFFFFFFu, n0 | n1)) {
-          push_candidate(n0, s0.pixel, place, q, cn, lane);
-          push_candidate(n1, s1.pixel, place + 32u, q, cn, lane);
-        }
-        if ((on | cn) >= 32u) drain_batches(q, on, cn, lane, tier2, candidate);
-      },
-      [&](uint32_t place, bool v0, bool v1) {
-        push_open(v0, place, q.open, on, lane);
-        push_open(v1, place + 32u, q.open, on, lane);
-        drain_batches(q, on, cn, lane, tier2, candidate);
-      },
-      mask);
+  // two points of a lane and their places
+  auto two_points = [&](const uint4& p0, const uint4& p1, uint32_t place0, uint32_t place1, bool v0, bool v1) {
+    ScreenTwo two = screen_two<kMode>(P, S, p0, p1, keys);
+    ScreenPoint &s0 = two.a, &s1 = two.b;
+    if constexpr (kFrom == kBandWords) {  // the last batch may be partial
+      s0.open &= v0;
+      s1.open &= v1;
+      if (!v0) s0.w = __int_as_float(0x7F800000);
+      if (!v1) s1.w = __int_as_float(0x7F800000);
+    }
+    if (__any_sync(0xFFFFFFFFu, s0.open | s1.open)) {
+      push_open(s0.open, place0, q.open, on, lane);
+      push_open(s1.open, place1, q.open, on, lane);
+    }
+    auto inside = [&](const ScreenPoint& o) {  // >= m: in the band; <= -m: outside it
+      return fminf(__fsub_rn(o.w, __fmaf_rn(o.k, S.lo_a, S.lo_b)), __fsub_rn(__fmaf_rn(o.k, S.hi_a, S.hi_b), o.w));
+    };
+    const float d0 = inside(s0), d1 = inside(s1);
+    add_push(d0 >= s0.m, s0.pixel, p0.w, aq, lane);
+    add_push(d1 >= s1.m, s1.pixel, p1.w, aq, lane);
+    add_drain_full(aq, accum, lane);
+    const bool n0 = fabsf(d0) < s0.m, n1 = fabsf(d1) < s1.m;
+    if (__any_sync(0xFFFFFFFFu, n0 | n1)) {
+      push_candidate(n0, s0.pixel, place0, q, cn, lane);
+      push_candidate(n1, s1.pixel, place1, q, cn, lane);
+    }
+    if ((on | cn) >= 32u) drain_batches(q, on, cn, lane, tier2, candidate);
+  };
+  const CloudSample sample = kFrom == kBandWords ? sample_cloud<kMode>(P, pts, n, T, lane) : CloudSample{false, false};
+  if (kFrom == kBandWords && sample.random)
+    band_points(pts, n, T, lane, reinterpret_cast<const uint2*>(mask),
+                reinterpret_cast<uint32_t*>(smem + kTableBytes + warps * (kAddRing * sizeof(uint2) + sizeof(PlaceQueues))) +
+                    warp * kBandQueue,
+                two_points);
+  else
+    screen_tiles<kFrom == kChunkMask>(
+        pts, n, T, lane,
+        [&](const uint4& p0, const uint4& p1, uint32_t place) { two_points(p0, p1, place, place + 32u, true, true); },
+        [&](uint32_t place, bool v0, bool v1) {
+          push_open(v0, place, q.open, on, lane);
+          push_open(v1, place + 32u, q.open, on, lane);
+          drain_batches(q, on, cn, lane, tier2, candidate);
+        },
+        mask);
   __syncwarp();
   if (cn) candidate(lane < cn ? lane : 0u, lane < cn);
   add_finish(aq, accum, lane);
@@ -569,7 +702,7 @@ struct ScreenLaunch {
 };
 
 constexpr size_t screen_smem(int warps, int tables, bool hq) {
-  return tables * kTableBytes + (size_t)warps * (hq ? sizeof(PlaceQueues) + kAddRing * sizeof(uint2) : sizeof(ScreenQueues));
+  return tables * kTableBytes + (size_t)warps * (hq ? sizeof(PlaceQueues) + kAddRing * sizeof(uint2) + kBandQueue * sizeof(uint32_t) : sizeof(ScreenQueues));
 }
 
 inline ScreenLaunch screen_launch(uint64_t n, int sms, int per_sm, int tables, bool hq) {
@@ -588,23 +721,28 @@ inline bool screen_opt_in(K kernel, int tables, bool hq) {
                               (int)screen_smem(kScreenThreads / 32, tables, hq)) == cudaSuccess;
 }
 
-template <int kMode>
+template <int kMode, bool kBand = false>
 inline void raster_screen_launch(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                                 unsigned long long* keys, int sms, int per_sm, cudaStream_t s) {
+                                 unsigned long long* keys, uint2* band, int sms, int per_sm, cudaStream_t s) {
   constexpr int most = kMode == kPiecewise ? kMaxRanges : kMode == kPiecewise2 ? 2 : 1;
-  static const bool opted = screen_opt_in(k_raster_screen<kMode>, most, false);
+  static const bool opted = screen_opt_in(k_raster_screen<kMode, kBand>, most, false);
   (void)opted;
   const ScreenLaunch L = screen_launch(n, sms, per_sm, table_blocks(P), false);
-  launch_after(k_raster_screen<kMode>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys);
+  launch_after(k_raster_screen<kMode, kBand>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, band);
 }
 
+// band (HQ frames of LINEAR or METRIC views, with the screen of pass 2's eps): receives the tiles' words for pass 2, or null.
 inline void launch_raster_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                                 unsigned long long* keys, int sms, int per_sm, cudaStream_t s) {
+                                 unsigned long long* keys, uint2* band, int sms, int per_sm, cudaStream_t s) {
   switch (screen_mode(P)) {
-    case kUnit256: return raster_screen_launch<kUnit256>(pts, n, P, S, keys, sms, per_sm, s);
-    case kUnit1: return raster_screen_launch<kUnit1>(pts, n, P, S, keys, sms, per_sm, s);
-    case kPiecewise2: return raster_screen_launch<kPiecewise2>(pts, n, P, S, keys, sms, per_sm, s);
-    case kPiecewise: return raster_screen_launch<kPiecewise>(pts, n, P, S, keys, sms, per_sm, s);
+    case kUnit256:
+      return band ? raster_screen_launch<kUnit256, true>(pts, n, P, S, keys, band, sms, per_sm, s)
+                  : raster_screen_launch<kUnit256>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+    case kUnit1:
+      return band ? raster_screen_launch<kUnit1, true>(pts, n, P, S, keys, band, sms, per_sm, s)
+                  : raster_screen_launch<kUnit1>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+    case kPiecewise2: return raster_screen_launch<kPiecewise2>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+    case kPiecewise: return raster_screen_launch<kPiecewise>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
   }
 }
 
@@ -624,16 +762,16 @@ struct HqScreenLaunch {
   void* args[9];
 };
 
-template <int kMode, bool kMask>
+template <int kMode, int kFrom>
 inline const void* hq_screen_kernel() {
-  static const bool opted = screen_opt_in(k_hq_screen<kMode, kMask>, 1, true);
+  static const bool opted = screen_opt_in(k_hq_screen<kMode, kFrom>, 1, true);
   (void)opted;
-  return reinterpret_cast<const void*>(k_hq_screen<kMode, kMask>);
+  return reinterpret_cast<const void*>(k_hq_screen<kMode, kFrom>);
 }
 
 inline void make_hq_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S, const unsigned long long* keys,
-                           unsigned long long* accum, uint32_t eps_num, uint32_t eps_den, const uint32_t* mask, int sms,
-                           int per_sm, HqScreenLaunch* o) {
+                           unsigned long long* accum, uint32_t eps_num, uint32_t eps_den, HqSource from,
+                           const uint32_t* mask, int sms, int per_sm, HqScreenLaunch* o) {
   o->pts = pts;
   o->n = n;
   o->P = P;
@@ -644,8 +782,9 @@ inline void make_hq_screen(const uint4* pts, uint64_t n, const CertParams& P, co
   o->eps_den = eps_den;
   o->mask = mask;
   const bool unit1 = screen_mode(P) == kUnit1;
-  o->kernel = mask ? (unit1 ? hq_screen_kernel<kUnit1, true>() : hq_screen_kernel<kUnit256, true>())
-                   : (unit1 ? hq_screen_kernel<kUnit1, false>() : hq_screen_kernel<kUnit256, false>());
+  o->kernel = from == kBandWords   ? (unit1 ? hq_screen_kernel<kUnit1, kBandWords>() : hq_screen_kernel<kUnit256, kBandWords>())
+              : from == kChunkMask ? (unit1 ? hq_screen_kernel<kUnit1, kChunkMask>() : hq_screen_kernel<kUnit256, kChunkMask>())
+                                   : (unit1 ? hq_screen_kernel<kUnit1, kAllTiles>() : hq_screen_kernel<kUnit256, kAllTiles>());
   o->shape = screen_launch(n, sms, per_sm, 1, true);
   void* args[9] = {&o->pts, &o->n, &o->P, &o->S, &o->keys, &o->accum, &o->eps_num, &o->eps_den, &o->mask};
   std::memcpy(o->args, args, sizeof(args));
@@ -670,7 +809,7 @@ inline void launch_raster_default(const uint4* pts, uint64_t n, const CertParams
                                   uint32_t* status, int sms, int per_sm, cudaStream_t s) {
   Screen S;
   if (make_screen(P, 0, 0, false, &S))
-    launch_raster_screen(pts, n, P, S, keys, sms, per_sm, s);
+    launch_raster_screen(pts, n, P, S, keys, nullptr, sms, per_sm, s);
   else
     raster_launch<false, false>(pts, n, P, keys, nullptr, status, sms, per_sm, s);
 }
@@ -684,11 +823,19 @@ inline void launch_hq_default(const uint4* pts, uint64_t n, const CertParams& P,
   if (band_bounds_exact(P.v.nq, eps_num, eps_den) && make_screen(P, eps_num, eps_den, !own_pass1, &S))
   {
     HqScreenLaunch l;
-    make_hq_screen(pts, n, P, S, keys, accum, eps_num, eps_den, nullptr, sms, per_sm, &l);
+    make_hq_screen(pts, n, P, S, keys, accum, eps_num, eps_den, kAllTiles, nullptr, sms, per_sm, &l);
     launch_hq_screen(l, s);
   }
   else
     hq_launch<false, false>(pts, n, P, keys, accum, eps_num, eps_den, status, sms, per_sm, s);
+}
+
+// Both passes of a frame over the same n points: whether pass 1 may leave pass 2 its words (enough tiles for the sample
+// that decides it), and the screen of both (eps at most 1: pass 1's margin holds pass 2's edge width).
+inline bool frame_screen(const CertParams& P, uint64_t n, int sms, int per_sm, uint32_t eps_num, uint32_t eps_den, Screen* S) {
+  const ScreenLaunch L = screen_launch(n, sms, per_sm, 1, false);
+  return n / kTile / ((uint64_t)L.grid * (L.threads / 32)) >= kSampleTiles && P.n_pw == 0 && eps_num <= eps_den && band_bounds_exact(P.v.nq, eps_num, eps_den) &&
+         make_screen(P, eps_num, eps_den, false, S);
 }
 
 // Pass 1 for a view with n >= 1 points. status: the framebuffer's status word (timeout bit).

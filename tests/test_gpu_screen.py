@@ -140,3 +140,36 @@ def test_projection_sizes(gpu, n, depth):
     got = [gpu.pcr_project_points(dev, RawView(np.asarray(v.view_proj), v.near, v.far, 320, 180, depth, 1000.0, ranges, t))
            for t in (0, 1)]
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("depth,scale", [(0, 1.0), (1, 1000.0)])
+def test_clouds_in_random_order(gpu, depth, scale):
+    """Enough tiles a warp that the passes sample the cloud and, in random order, pass 1 leaves pass 2 its words: at eps up
+    to 1, on a second frame, after a smaller cloud, with bands above 1 (without words), and captured."""
+    import torch
+    n = 97 * 152 * 8 * 64 + 4321
+    pts = scenes.lidar(n, 49)
+    scenes.shuffle(pts, 2)
+    dev, v = _dev(pts), scenes.lidar_1km_view(400, 225)
+    one = {"blocks_per_sm": 1}
+    for eps in ((1, 100), (1, 1), (3, 2), (0, 1)):
+        want = _frames(gpu, dev, v, depth, scale, eps, tuning=one)
+        fb = gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ)
+        gpu.pcr_set_tuning(fb, **one)
+        view = _view(v, depth, scale)
+        keys, acc = gpu.pcr_framebuffer_keys(fb)
+        for points in (dev, dev[:300_001], dev):
+            gpu.pcr_clear(fb)
+            gpu.pcr_render_hq_splat(fb, points, view, *eps)
+        assert torch.equal(keys, want[0]) and torch.equal(acc, want[1])
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            gpu.pcr_clear(fb)
+            gpu.pcr_render_hq_splat(fb, dev, view, *eps)
+        acc.fill_(5)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(keys, want[0]) and torch.equal(acc, want[1])
+        del graph
+        fb.close()
