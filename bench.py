@@ -140,10 +140,10 @@ def _code_only(text: str) -> str:
 
 
 def _csrc_digest() -> str:
-    """Digest of the code (comments and layout aside) that defines the two point-pass kernels (k_raster_cert,
-    k_hq_cert)."""
+    """Digest of the code (comments and layout aside) that defines the two point-pass kernels of default tuning
+    (k_raster_screen, k_hq_screen)."""
     h = hashlib.sha256()
-    for name in ("pcr_certified.cuh", "pcr_device.cuh", "pcr_kernels.cuh"):
+    for name in ("pcr_certified.cuh", "pcr_device.cuh", "pcr_kernels.cuh", "pcr_screen.cuh"):
         f = os.path.join(ROOT, "paper_1908_02681_gb300", "csrc", name)
         with open(f, encoding="utf-8") as fh:
             h.update(name.encode() + _code_only(fh.read()).encode())
@@ -234,7 +234,7 @@ def _config(wl, args, n, world=1):
 
 
 # The reference arm's work bound: point-frames over the whole run (warm-up included), about 50 s of the
-# oracle on one Grace core. The driver's short runs (about 25 frames) then take the full workload.
+# oracle on one Grace core. Short runs (about 25 frames) then take the full workload.
 REFERENCE_POINT_FRAMES = 3_000_000_000
 
 
