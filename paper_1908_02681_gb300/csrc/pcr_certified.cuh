@@ -35,6 +35,7 @@
 // The output is therefore bit-identical to the FP64 definition.
 #pragma once
 
+#include <atomic>
 #include <cmath>
 #include <cstring>
 
@@ -1543,6 +1544,20 @@ inline int resident_blocks(K kernel) {
   return b;
 }
 
+// Opts a kernel in to `bytes` of dynamic shared memory, once per device (the attribute belongs to the current device).
+// `done`: the kernel's own set of devices.
+template <typename K>
+inline cudaError_t opt_in_shared(K kernel, size_t bytes, std::atomic<uint64_t>& done) {
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = device < 64 ? 1ull << device : 0ull;
+  if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
+
 // Grid of a persistent grid-stride launch: never more blocks than can be resident at once.
 inline unsigned persistent_grid(int resident, uint64_t n, int sms, int per_sm) {
   return cert_grid(n, sms, per_sm < resident ? per_sm : resident);
@@ -1555,9 +1570,8 @@ inline void raster_launch5(const uint4* pts, uint64_t n, const CertParams& P, un
   auto kernel = k_raster_cert<kApprox, kMerge, kStats, kRing, kPw, kBand>;
   if constexpr (kPw) {
     // the ranges' tables in dynamic shared memory: up to kMaxRanges * 12 KB (opt in above 48 KB once)
-    static const bool opted = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)(kMaxRanges * kTableBytes)) == cudaSuccess;
-    (void)opted;
+    static std::atomic<uint64_t> opted{0};
+    opt_in_shared(kernel, kMaxRanges * kTableBytes, opted);
     const size_t dyn = (size_t)P.n_pw * kTableBytes;
     int resident = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kCertThreads, dyn) != cudaSuccess ||

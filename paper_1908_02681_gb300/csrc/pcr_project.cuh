@@ -87,10 +87,9 @@ inline cudaError_t launch_project(const uint4* pts, uint64_t n, const CertParams
                                   int sms, cudaStream_t s) {
   constexpr int most_tables = kPw ? kMaxRanges : 1;
   constexpr size_t queue = kCand * sizeof(uint32_t);
-  static const cudaError_t opted =
-      cudaFuncSetAttribute(k_project_cert<kPw>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(most_tables * kTableBytes + kScreenThreads / 32 * queue));
-  if (opted != cudaSuccess) return opted;
+  static std::atomic<uint64_t> opted{0};
+  const cudaError_t e = opt_in_shared(k_project_cert<kPw>, most_tables * kTableBytes + kScreenThreads / 32 * queue, opted);
+  if (e != cudaSuccess) return e;
   const ScreenLaunch L = screen_launch(n, sms, kScreenThreads / 256, 1, false);
   launch_after(k_project_cert<kPw>, L.grid, L.threads, table_blocks(P) * kTableBytes + L.threads / 32 * queue, s, pts, n, P,
                pix, key);

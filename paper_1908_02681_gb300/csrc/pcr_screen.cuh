@@ -461,11 +461,11 @@ __device__ __forceinline__ void band_points(const uint4* __restrict__ pts, uint6
 }
 
 // Pass 1 (Section 2.1), exact transform. Issue slots and the latency of the stored-key reads
-// bound it (61 % busy and the top stall at 20M points). 32 warps an SM at 64 registers, as one block: 48 warps with one
+// bound it (67 % busy and the top stall at 20M points). 32 warps an SM at 64 registers, as one block: 48 warps with one
 // point a lane (40 registers) and 24 warps (80) were slower, and one block holds one table, which leaves L1 more room
 // for the keys in flight than two of 512 threads (shuffled 37M points, both passes 0.44 against 0.57 ms). Against
-// k_raster_cert, which computes every point's code, on one GB300: 400M city points at 4K 2.23 to 1.41 ms (the culled
-// points), 37M shuffled 0.227 to 0.18, 100M in scan order 0.539 to 0.51, and frames of 0.5 to 4 points per pixel equal
+// k_raster_cert, which computes every point's code, on one GB300: 400M city points at 4K 2.23 to 1.10 ms (the culled
+// points), 37M shuffled 0.227 to 0.18, 100M in scan order 0.539 to 0.48, and frames of 0.5 to 4 points per pixel equal
 // or a few per cent faster, so it runs at every size.
 // kBand (HQ frames): also writes, per tile, a bit for each point that pass 2 may accept: clear where the point is culled or
 // certainly beyond the upper band edge of the key its pixel holds (a stored key only decreases, and the edge with it).
@@ -714,19 +714,12 @@ inline ScreenLaunch screen_launch(uint64_t n, int sms, int per_sm, int tables, b
                       screen_smem(warps, tables, hq)};
 }
 
-// Opts a screened kernel in to its largest shared memory.
-template <typename K>
-inline bool screen_opt_in(K kernel, int tables, bool hq) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)screen_smem(kScreenThreads / 32, tables, hq)) == cudaSuccess;
-}
-
 template <int kMode, bool kBand = false>
 inline void raster_screen_launch(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
                                  unsigned long long* keys, uint2* band, int sms, int per_sm, cudaStream_t s) {
   constexpr int most = kMode == kPiecewise ? kMaxRanges : kMode == kPiecewise2 ? 2 : 1;
-  static const bool opted = screen_opt_in(k_raster_screen<kMode, kBand>, most, false);
-  (void)opted;
+  static std::atomic<uint64_t> opted{0};
+  opt_in_shared(k_raster_screen<kMode, kBand>, screen_smem(kScreenThreads / 32, most, false), opted);
   const ScreenLaunch L = screen_launch(n, sms, per_sm, table_blocks(P), false);
   launch_after(k_raster_screen<kMode, kBand>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, band);
 }
@@ -764,8 +757,8 @@ struct HqScreenLaunch {
 
 template <int kMode, int kFrom>
 inline const void* hq_screen_kernel() {
-  static const bool opted = screen_opt_in(k_hq_screen<kMode, kFrom>, 1, true);
-  (void)opted;
+  static std::atomic<uint64_t> opted{0};
+  opt_in_shared(k_hq_screen<kMode, kFrom>, screen_smem(kScreenThreads / 32, 1, true), opted);
   return reinterpret_cast<const void*>(k_hq_screen<kMode, kFrom>);
 }
 
