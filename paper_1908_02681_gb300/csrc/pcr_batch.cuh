@@ -149,6 +149,7 @@ struct BatchTuning {
                               // 2: one single-view pass per view
   int slice_words = 1;        // mask words (32 chunks each) per work item: 1, 2 or 4
   int points_per_thread = 1;  // points a thread classifies per step: 1 or 2
+  bool auto_points = true;    // not chosen by the caller: pass 1 takes 2 (see batch_points)
   int blocks_per_sm = 4;      // capped at the blocks that can be resident
   int merge_width = 0;        // 0: one atomic per fragment; 8, 16 or 32: same-pixel fragments of that many
                               // lanes merged first
@@ -308,6 +309,13 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
 // block: 0.49, 8: 0.46), 20M unchanged.
 constexpr int kMinItems = 4;
 
+// Points a thread takes per step. Unless the caller chose, pass 1 takes 2, whose key reads are in flight together: 16
+// views of mixed sizes on one GB300, 1 and 2 points: 1M points 327 and 321 us, 6M 769 and 747, 20M 1888 and 1818.
+template <bool kHq>
+inline int batch_points(const BatchTuning& t) {
+  return t.auto_points ? (kHq ? 1 : 2) : t.points_per_thread;
+}
+
 // Launches the batch pass kernel of a tuning (template instance by merging and points per thread).
 template <bool kHq>
 inline void batch_pass_launch(const BatchTuning& t, int sms, int resident, const uint4* pts, uint64_t n,
@@ -324,9 +332,9 @@ inline void batch_pass_launch(const BatchTuning& t, int sms, int resident, const
   k_batch_pass<kHq, M, K><<<grid, kCertThreads, 0, s>>>(pts, n, params, tables, slots, masks, n_views, n_chunks, \
                                                         next_item, eps_num, eps_den, sc, mw)
   if (t.merge_width > 0) {
-    if (t.points_per_thread == 2) PCR_BATCH_LAUNCH(true, 2); else PCR_BATCH_LAUNCH(true, 1);
+    if (batch_points<kHq>(t) == 2) PCR_BATCH_LAUNCH(true, 2); else PCR_BATCH_LAUNCH(true, 1);
   } else {
-    if (t.points_per_thread == 2) PCR_BATCH_LAUNCH(false, 2); else PCR_BATCH_LAUNCH(false, 1);
+    if (batch_points<kHq>(t) == 2) PCR_BATCH_LAUNCH(false, 2); else PCR_BATCH_LAUNCH(false, 1);
   }
 #undef PCR_BATCH_LAUNCH
 }
@@ -337,11 +345,11 @@ inline int batch_pass_resident(const BatchTuning& t) {
   int b = 0;
   cudaError_t e;
   if (t.merge_width > 0)
-    e = t.points_per_thread == 2
+    e = batch_points<kHq>(t) == 2
             ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, true, 2>, kCertThreads, 0)
             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, true, 1>, kCertThreads, 0);
   else
-    e = t.points_per_thread == 2
+    e = batch_points<kHq>(t) == 2
             ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, false, 2>, kCertThreads, 0)
             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, false, 1>, kCertThreads, 0);
   if (e != cudaSuccess || b < 1) {
