@@ -326,8 +326,10 @@ pcr_status pcr_batch_set_views(pcr_batch* batch, const pcr_view* views);
  *     turn for every view (so each range is read from HBM once), then pass 2 (hq) likewise, or, for clouds of at
  *     least 2.5 * 10^6 points, one launch per view that skips the view's culled chunks. A frame of at
  *     most 4 views, or of a cloud of at least 10^8 points, instead runs one single-view pass per view,
- *     which is faster there (frames recorded by pcr_batch_capture always use the persistent launch);
+ *     which is faster there (never under stream capture: the persistent launch reads the views from device memory);
  *   - resolve every framebuffer into its output (and clear it, see pcr_batch_create).
+ * Under a stream capture of the caller's, both passes of the frame use the persistent launch, and replays of that graph
+ * draw the views set since (with route 2 of pcr_batch_tuning the views at the capture).
  * Framebuffer contents equal those of pcr_render_atomicmin / pcr_render_hq_splat per view, bit for bit. */
 pcr_status pcr_batch_render(pcr_batch* batch, pcr_stream_t stream);
 
