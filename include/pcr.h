@@ -314,8 +314,8 @@ pcr_status pcr_batch_create(pcr_cloud* cloud, pcr_framebuffer* const* fbs, uint3
                             int32_t clear_after, pcr_batch** out);
 
 /* Sets the views of the next frames (count of them). Every view must use LINEAR or METRIC depth within
- * the single-precision preconditions (every perspective lookAt camera does), else PCR_ERR_INVALID_ARG.
- * Blocks until the previous frame has copied the earlier views to the device. */
+ * the single-precision preconditions (every perspective lookAt camera does), else PCR_ERR_INVALID_ARG and
+ * the views set before stay. Blocks until the previous frame has copied the earlier views to the device. */
 pcr_status pcr_batch_set_views(pcr_batch* batch, const pcr_view* views);
 
 /* Enqueues one frame on `stream`:

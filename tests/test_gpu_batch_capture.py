@@ -98,3 +98,31 @@ def test_beside_the_batch_s_own_frame(gpu):
     gpu.pcr_batch_launch(s.batch, own)
     s.check(s.views(6))
     s.batch.close()
+
+
+@pytest.mark.parametrize("bad", [0, 1, 5])
+def test_refused_views_leave_the_staged_frame(gpu, bad):
+    """A set of views of which one is refused (near beyond far) changes nothing: un-captured frames and the batch's
+    own captured frame stay those of the views before, also where the screened pass 2 cannot take those (depth codes in
+    units of 1e26 m)."""
+    import torch
+    from tests.helpers import RawView
+    s = Setup(gpu)
+    own = torch.cuda.Stream()
+    for k, scale in enumerate((None, 1e-26)):
+        good = s.views(3 + k)
+        if scale:
+            good = [RawView(v.view_proj, v.near, v.far, v.width, v.height, 1, scale) for v in good]
+        gpu.pcr_batch_set_views(s.batch, good)
+        if not k:
+            gpu.pcr_batch_capture(s.batch, own)
+        refused = s.views(9)
+        refused[bad] = RawView(refused[bad].view_proj, 10.0, 1.0, refused[bad].width, refused[bad].height)
+        for _ in range(2):
+            with pytest.raises(gpu.PcrError):
+                gpu.pcr_batch_set_views(s.batch, refused)
+            gpu.pcr_batch_render(s.batch)
+            s.check(good)
+            gpu.pcr_batch_launch(s.batch, own)
+            s.check(good)
+    s.batch.close()
