@@ -126,3 +126,27 @@ def test_refused_views_leave_the_staged_frame(gpu, bad):
             gpu.pcr_batch_launch(s.batch, own)
             s.check(good)
     s.batch.close()
+
+
+@pytest.mark.parametrize("own", [False, True])
+def test_views_wait_for_a_replay_s_copy(gpu, own):
+    """pcr_batch_set_views waits until a replay that is still queued (behind 50 ms of other work) has copied its views,
+    also where the graph is the caller's."""
+    import torch
+    s = Setup(gpu, False, 300_001)
+    gpu.pcr_batch_set_views(s.batch, s.views(3))
+    stream = torch.cuda.Stream()
+    if own:
+        gpu.pcr_batch_capture(s.batch, stream)
+    else:
+        graph = s.capture()
+    for seed in range(3, 7):
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(100_000_000)
+            if own:
+                gpu.pcr_batch_launch(s.batch, stream)
+            else:
+                graph.replay()
+        gpu.pcr_batch_set_views(s.batch, s.views(seed + 1))
+        s.check(s.views(seed))
+    s.batch.close()
