@@ -118,7 +118,9 @@ typedef struct {
                                in random order (pass 2 about 17 % faster, the HQ frame about 5 %), not in scan
                                order, where pass 1's extra work outweighs it; the autotuner tries both. The first
                                recording of n points allocates n / 8 bytes of device memory (not during stream
-                               capture, where nothing is recorded); a clear drops the record. */
+                               capture, where nothing is recorded beyond the memory that is there; memory that a
+                               captured frame uses is kept when a larger frame outgrows it); a clear drops the
+                               record. */
   uint32_t band_eps_num, band_eps_den; /* eps of the records (default 1 / 100); band_eps_den in 1..2^20 */
   int32_t band_bounds;      /* 1: pass 2 with the exact transform first turns each pixel's qmin into its accept
                                bounds {qmin, qmin + floor(eps_num * (qmin + Nq) / eps_den)} (one more kernel,

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -17,6 +18,12 @@
 #include "pcr_kernels.cuh"
 #include "pcr_project.cuh"
 #include "pcr_screen.cuh"
+
+// A band mask that was outgrown while a captured frame may still use it: kept until the framebuffer goes.
+struct KeptMask {
+  uint32_t* mask;
+  KeptMask* next;
+};
 
 struct pcr_framebuffer {
   int32_t width, height;
@@ -35,6 +42,8 @@ struct pcr_framebuffer {
   // points, count, view and eps of the pass 1 that wrote it, until the framebuffer is cleared
   uint32_t* band_mask;
   uint64_t band_words;
+  bool band_captured;   // a captured frame holds the mask's address
+  KeptMask* kept_masks;
   bool band_valid;
   const void* band_pts;
   uint64_t band_n;
@@ -175,23 +184,32 @@ struct BandRequest {
 bool band_reserve(pcr_framebuffer* fb, uint64_t n_total, cudaStream_t s) {
   fb->band_valid = false;
   const uint64_t words = 2 * ((n_total + pcr::kTile - 1) / pcr::kTile);
-  if (words <= fb->band_words) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
+  const bool captured = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (captured) cudaGetLastError();
+  if (words <= fb->band_words) {
+    fb->band_captured = fb->band_captured || captured;
+    return true;
   }
+  if (captured) return false;
+  KeptMask* keep = nullptr;
+  if (fb->band_captured && !(keep = new (std::nothrow) KeptMask)) return false;
   uint32_t* m = nullptr;
   if (cudaMalloc(&m, words * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();
+    delete keep;
     return false;
   }
-  if (fb->band_mask) {
+  if (keep) {  // its replays go on writing and reading the old mask
+    *keep = KeptMask{fb->band_mask, fb->kept_masks};
+    fb->kept_masks = keep;
+  } else if (fb->band_mask) {
     cudaStreamSynchronize(s);  // the old mask may still be read by pass 2 on this stream
     cudaFree(fb->band_mask);
   }
   fb->band_mask = m;
   fb->band_words = words;
+  fb->band_captured = false;
   return true;
 }
 
@@ -373,6 +391,11 @@ pcr_status pcr_destroy_framebuffer(pcr_framebuffer* fb) {
   cudaFree(fb->bounds);
   cudaFree(fb->status);
   cudaFree(fb->band_mask);
+  while (KeptMask* k = fb->kept_masks) {
+    fb->kept_masks = k->next;
+    cudaFree(k->mask);
+    delete k;
+  }
   for (cudaEvent_t e : fb->copy_events)
     if (e) cudaEventDestroy(e);
   cudaSetDevice(prev);

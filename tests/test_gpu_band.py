@@ -191,3 +191,37 @@ def test_band_records_across_eps(gpu, eps, metric):
     assert np.array_equal(gpu.keys_to_numpy(keys), ref)
     _expect(gpu, fb, pts, view, ref, eps)
     fb.close()
+
+
+def test_records_of_a_captured_frame_outlive_a_larger_frame(gpu):
+    """A captured frame keeps the memory of its records when a larger frame needs more: its replays draw the same frame and
+    write nothing that was allocated since."""
+    import torch
+    pts = scenes.lidar(2_000_003, 88)
+    scenes.shuffle(pts, 10)
+    dev, more = _dev(pts), _dev(scenes.lidar(6_000_001, 89))
+    view = scenes.lidar_1km_view(640, 360)
+    fb = gpu.pcr_create_framebuffer(view.width, view.height, gpu.PCR_FB_HQ)
+    gpu.pcr_set_tuning(fb, 0, 8, 0, band_filter=1, band_eps=(1, 100))
+    gpu.pcr_render_hq_splat(fb, dev, view)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gpu.pcr_clear(fb)
+        gpu.pcr_render_hq_splat(fb, dev, view)
+    others = []
+    for _ in range(2):
+        gpu.pcr_clear(fb)
+        gpu.pcr_render_hq_splat(fb, more, view)
+        # framebuffers whose keys are as large as the first frame's records
+        others += [gpu.pcr_create_framebuffer(15626, 2) for _ in range(4)]
+        graph.replay()
+    keys, _ = gpu.pcr_framebuffer_keys(fb)
+    ref = oracle.render_atomicmin(pts, view)
+    assert np.array_equal(gpu.keys_to_numpy(keys), ref)
+    _expect(gpu, fb, pts, view, ref)
+    for o in others:
+        assert bool((gpu.pcr_framebuffer_keys(o)[0] == -1).all())
+    torch.cuda.synchronize()
+    del graph
+    fb.close()
