@@ -204,9 +204,9 @@ pcr_status pcr_project_points(const pcr_point* d_points, uint64_t n, const pcr_v
  * Requirements: fb created with PCR_FB_HQ, and cleared; depth_mode LINEAR or METRIC; 1 <= eps_den <= 2^20;
  * eps_num * (2^40 + Nq) < 2^64. Colour sums are u32 per channel: valid while every pixel gets at most 2^24
  * contributing fragments (checked by the HQ resolve, reported as PCR_ERR_OVERFLOW). pcr_tuning.band_bounds
- * selects how pass 2 evaluates the test; the result is the same. With default tuning, the first call of 3 * 10^7 points
- * or more allocates n / 8 bytes of device memory on fb (not during stream capture), in which pass 1 tells pass 2 which
- * points of a cloud in random order it may accept. */
+ * selects how pass 2 evaluates the test; the result is the same. With default tuning, a call of 3 * 10^7 points or
+ * more that follows one whose points came in random order allocates n / 8 bytes of device memory on fb, once (not during
+ * stream capture), in which pass 1 tells pass 2 which points it may accept. */
 pcr_status pcr_render_hq_splat(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr_view* view,
                                uint32_t eps_num, uint32_t eps_den, pcr_stream_t stream);
 

@@ -44,6 +44,7 @@ struct pcr_framebuffer {
   uint64_t band_words;
   bool band_captured;   // a captured frame holds the mask's address
   KeptMask* kept_masks;
+  volatile uint32_t* random_hint;  // HQ: written by pass 1 of large frames (see take_hint), or null
   bool band_valid;
   const void* band_pts;
   uint64_t band_n;
@@ -171,6 +172,37 @@ pcr_status after_launch(const char* what, uint64_t launches = 1) {
   return e == cudaSuccess ? PCR_OK : cuda_fail(e, what);
 }
 
+// One word of pinned host memory per HQ framebuffer, in which pass 1 of a large frame leaves whether it found the cloud in
+// random order; a later frame reads it without waiting for anything. From one page for the process (null when its words
+// are all taken or it cannot be had).
+constexpr int kHints = 1024;
+std::mutex g_hint_mu;
+uint32_t* g_hint_page = nullptr;
+bool g_hint_taken[kHints] = {};
+
+volatile uint32_t* take_hint() {
+  std::lock_guard<std::mutex> lock(g_hint_mu);
+  if (!g_hint_page && cudaHostAlloc((void**)&g_hint_page, kHints * sizeof(uint32_t),
+                                    cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    g_hint_page = nullptr;
+    return nullptr;
+  }
+  for (int i = 0; i < kHints; ++i)
+    if (!g_hint_taken[i]) {
+      g_hint_taken[i] = true;
+      g_hint_page[i] = 0u;
+      return g_hint_page + i;
+    }
+  return nullptr;
+}
+
+void give_hint(volatile uint32_t* hint) {
+  if (!hint) return;
+  std::lock_guard<std::mutex> lock(g_hint_mu);
+  g_hint_taken[hint - g_hint_page] = false;
+}
+
 // A band mask request for pass 1: on, its eps, and where the launch's first tile sits in the mask (a pass 1
 // over a tile-aligned part of the frame's points).
 struct BandRequest {
@@ -274,20 +306,19 @@ ulonglong2* bounds_buffer(pcr_framebuffer* fb, cudaStream_t s) {
   return fb->bounds;
 }
 
-// A frame whose two passes run here with default tuning (fb's band mask holds pass 1's words for pass 2, see
-// k_raster_screen): the screen of both, or false (then the passes run without). Not under capture: the buffer may grow, and
-// a replay would write the old one.
-bool frame_words(pcr_framebuffer* fb, uint64_t n, const pcr::DevView& dv, int transform, uint32_t eps_num, uint32_t eps_den,
-                 cudaStream_t s, const pcr::CertParams** P, pcr::Screen* S) {
+// A frame of default tuning that is large enough for its passes to sample the cloud (see frame_screen): the screen of both.
+// Not under capture: the words' memory may grow, and a replay would write the old one.
+bool frame_samples(pcr_framebuffer* fb, uint64_t n, const pcr::DevView& dv, int transform, uint32_t eps_num, uint32_t eps_den,
+                   cudaStream_t s, const pcr::CertParams** P, pcr::Screen* S) {
   const pcr::Tuning& t = fb->tuning;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return false;
   }
-  return transform == PCR_TRANSFORM_EXACT && !t.merge && !t.staging && !t.band_filter &&
-         !t.band_bounds && pcr::cached_cert(dv, false, P) && pcr::frame_screen(**P, n, sm_count(fb->device), t.blocks_per_sm, eps_num, eps_den, S) &&
-         band_reserve(fb, n, s);
+  return transform == PCR_TRANSFORM_EXACT && !t.merge && !t.staging && !t.band_filter && !t.band_bounds &&
+         pcr::cached_cert(dv, false, P) &&
+         pcr::frame_screen(**P, n, sm_count(fb->device), t.blocks_per_sm, eps_num, eps_den, S);
 }
 
 pcr_status launch_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n, const pcr::DevView& dv,
@@ -314,13 +345,17 @@ pcr_status render_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n,
                      uint32_t eps_num, uint32_t eps_den, cudaStream_t s) {
   const pcr::CertParams* P = nullptr;
   pcr::Screen S;
-  if (frame_words(fb, n, dv, transform, eps_num, eps_den, s, &P, &S)) {
+  if (frame_samples(fb, n, dv, transform, eps_num, eps_den, s, &P, &S)) {
     const uint4* pts = reinterpret_cast<const uint4*>(d_points);
     const int sms = sm_count(fb->device), per_sm = fb->tuning.blocks_per_sm;
-    pcr::launch_raster_screen(pts, n, *P, S, fb->keys, reinterpret_cast<uint2*>(fb->band_mask), sms, per_sm, s);
+    // memory for pass 1's words only once a frame has found its cloud in random order: in scan order they are not written,
+    // and the allocation takes 95 us (first frame of a framebuffer, 100M scanned points: 1034 us with it, 938 without)
+    const bool words = fb->random_hint && *fb->random_hint && band_reserve(fb, n, s);
+    pcr::launch_raster_screen(pts, n, *P, S, fb->keys, words ? reinterpret_cast<uint2*>(fb->band_mask) : nullptr,
+                              const_cast<uint32_t*>(fb->random_hint), sms, per_sm, s);
     pcr::HqScreenLaunch l;
     pcr::make_hq_screen(pts, n, *P, S, fb->keys, reinterpret_cast<unsigned long long*>(fb->accum), eps_num, eps_den,
-                        pcr::kBandWords, fb->band_mask, sms, per_sm, &l);
+                        words ? pcr::kBandWords : pcr::kAllTiles, words ? fb->band_mask : nullptr, sms, per_sm, &l);
     pcr::launch_hq_screen(l, s);
     return after_launch("screened frame", 2);
   }
@@ -364,6 +399,7 @@ pcr_status pcr_create_framebuffer(int32_t width, int32_t height, uint32_t flags,
     return e == cudaErrorMemoryAllocation ? fail(PCR_ERR_OOM, "cudaMalloc of %llu pixels failed", (unsigned long long)npx)
                                           : cuda_fail(e, "cudaMalloc");
   }
+  if (flags & PCR_FB_HQ) fb->random_hint = take_hint();
   e = cudaMemset(fb->status, 0, 256);
   if (e == cudaSuccess) {
     pcr::k_clear<<<grid_for(npx / 2 + 1, 256, fb->device, 4), 256>>>(fb->keys, fb->accum, npx);
@@ -398,6 +434,7 @@ pcr_status pcr_destroy_framebuffer(pcr_framebuffer* fb) {
   }
   for (cudaEvent_t e : fb->copy_events)
     if (e) cudaEventDestroy(e);
+  give_hint(fb->random_hint);
   cudaSetDevice(prev);
   delete fb;
   return PCR_OK;

@@ -467,12 +467,13 @@ __device__ __forceinline__ void band_points(const uint4* __restrict__ pts, uint6
 // k_raster_cert, which computes every point's code, on one GB300: 400M city points at 4K 2.23 to 1.10 ms (the culled
 // points), 37M shuffled 0.227 to 0.18, 100M in scan order 0.539 to 0.48, and frames of 0.5 to 4 points per pixel equal
 // or a few per cent faster, so it runs at every size.
+// hint (HQ frames, or null): receives whether the sample found the cloud in random order.
 // kBand (HQ frames): also writes, per tile, a bit for each point that pass 2 may accept: clear where the point is culled or
 // certainly beyond the upper band edge of the key its pixel holds (a stored key only decreases, and the edge with it).
 template <int kMode, bool kBand>
 __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P, const __grid_constant__ Screen S,
-    unsigned long long* __restrict__ keys, uint2* __restrict__ band) {
+    unsigned long long* __restrict__ keys, uint2* __restrict__ band, uint32_t* __restrict__ hint) {
   extern __shared__ __align__(16) unsigned char smem[];
   long long* const sF = reinterpret_cast<long long*>(smem);
   const int tables = kMode >= kPiecewise2 ? P.n_pw : 1;
@@ -483,6 +484,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
   build_tables(P.col, tables, sF);
   wait_previous();
   const CloudSample sample = sample_cloud<kMode>(P, pts, n, T, lane);
+  if (kMode < kPiecewise2 && hint && T.g == 0u && lane == 0u) *hint = sample.random ? 1u : 0u;
   uint32_t cn = 0, on = 0;
   auto tier2 = [&](uint32_t place) { raster_deferred(P, sF, point_at(pts, T, place), keys); };
   auto commit = [&](bool need, const uint4& p, uint32_t pixel, uint32_t place) {
@@ -716,26 +718,28 @@ inline ScreenLaunch screen_launch(uint64_t n, int sms, int per_sm, int tables, b
 
 template <int kMode, bool kBand = false>
 inline void raster_screen_launch(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                                 unsigned long long* keys, uint2* band, int sms, int per_sm, cudaStream_t s) {
+                                 unsigned long long* keys, uint2* band, uint32_t* hint, int sms, int per_sm, cudaStream_t s) {
   constexpr int most = kMode == kPiecewise ? kMaxRanges : kMode == kPiecewise2 ? 2 : 1;
   static std::atomic<uint64_t> opted{0};
   opt_in_shared(k_raster_screen<kMode, kBand>, screen_smem(kScreenThreads / 32, most, false), opted);
   const ScreenLaunch L = screen_launch(n, sms, per_sm, table_blocks(P), false);
-  launch_after(k_raster_screen<kMode, kBand>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, band);
+  launch_after(k_raster_screen<kMode, kBand>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, band, hint);
 }
 
 // band (HQ frames of LINEAR or METRIC views, with the screen of pass 2's eps): receives the tiles' words for pass 2, or null.
+// hint: see k_raster_screen.
 inline void launch_raster_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                                 unsigned long long* keys, uint2* band, int sms, int per_sm, cudaStream_t s) {
+                                 unsigned long long* keys, uint2* band, uint32_t* hint, int sms, int per_sm,
+                                 cudaStream_t s) {
   switch (screen_mode(P)) {
     case kUnit256:
-      return band ? raster_screen_launch<kUnit256, true>(pts, n, P, S, keys, band, sms, per_sm, s)
-                  : raster_screen_launch<kUnit256>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+      return band ? raster_screen_launch<kUnit256, true>(pts, n, P, S, keys, band, hint, sms, per_sm, s)
+                  : raster_screen_launch<kUnit256>(pts, n, P, S, keys, nullptr, hint, sms, per_sm, s);
     case kUnit1:
-      return band ? raster_screen_launch<kUnit1, true>(pts, n, P, S, keys, band, sms, per_sm, s)
-                  : raster_screen_launch<kUnit1>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
-    case kPiecewise2: return raster_screen_launch<kPiecewise2>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
-    case kPiecewise: return raster_screen_launch<kPiecewise>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+      return band ? raster_screen_launch<kUnit1, true>(pts, n, P, S, keys, band, hint, sms, per_sm, s)
+                  : raster_screen_launch<kUnit1>(pts, n, P, S, keys, nullptr, hint, sms, per_sm, s);
+    case kPiecewise2: return raster_screen_launch<kPiecewise2>(pts, n, P, S, keys, nullptr, nullptr, sms, per_sm, s);
+    case kPiecewise: return raster_screen_launch<kPiecewise>(pts, n, P, S, keys, nullptr, nullptr, sms, per_sm, s);
   }
 }
 
@@ -802,7 +806,7 @@ inline void launch_raster_default(const uint4* pts, uint64_t n, const CertParams
                                   uint32_t* status, int sms, int per_sm, cudaStream_t s) {
   Screen S;
   if (make_screen(P, 0, 0, false, &S))
-    launch_raster_screen(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+    launch_raster_screen(pts, n, P, S, keys, nullptr, nullptr, sms, per_sm, s);
   else
     raster_launch<false, false>(pts, n, P, keys, nullptr, status, sms, per_sm, s);
 }

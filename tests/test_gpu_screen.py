@@ -173,3 +173,40 @@ def test_clouds_in_random_order(gpu, depth, scale):
         assert torch.equal(keys, want[0]) and torch.equal(acc, want[1])
         del graph
         fb.close()
+
+
+def test_words_memory_only_after_random_order(gpu):
+    """The memory of pass 1's words is taken by the frame after one that found its cloud in random order, not by frames in
+    scan order; the frames are the same before and after."""
+    import torch
+    n = 20_000_003
+    pts = scenes.lidar(n, 50)
+    scan = _dev(pts)
+    scenes.shuffle(pts, 3)
+    v, one = scenes.lidar_1km_view(400, 225), {"blocks_per_sm": 1}
+    view = _view(v)
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    def frame(fb, points):
+        gpu.pcr_clear(fb)
+        gpu.pcr_render_hq_splat(fb, points, view)
+        return tuple(t.clone() for t in gpu.pcr_framebuffer_keys(fb))
+
+    for order in ("warm-up", "scan", "shuffled"):
+        points = scan if order == "scan" else _dev(pts)
+        want = _frames(gpu, points, v, 0, 1.0, (1, 100), tuning=one)
+        fb = gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ)
+        gpu.pcr_set_tuning(fb, **one)
+        frame(fb, points[:100_000])  # its results' memory is taken
+        left = [free()]
+        for _ in range(3):
+            got = frame(fb, points)
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+            left.append(free())
+        if order != "warm-up":
+            assert left[1] == left[0] and left[3] == left[2]
+            assert (left[2] < left[1]) == (order == "shuffled")
+        fb.close()
