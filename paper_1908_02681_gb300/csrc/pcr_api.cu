@@ -211,6 +211,14 @@ struct BandRequest {
   uint64_t tile_offset = 0;
 };
 
+// While it lives, this thread may allocate and free although a capture is in progress elsewhere: memory that belongs to no
+// graph, whose allocation would otherwise fail and break a capture in the global mode (cudaStreamBeginCapture).
+struct OutsideCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~OutsideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Makes the framebuffer's band mask hold `n_total` points (grown with cudaMalloc outside stream capture only);
 // false when it cannot (then pass 1 writes no mask). The mask stops describing any points.
 bool band_reserve(pcr_framebuffer* fb, uint64_t n_total, cudaStream_t s) {
@@ -226,6 +234,7 @@ bool band_reserve(pcr_framebuffer* fb, uint64_t n_total, cudaStream_t s) {
   if (captured) return false;
   KeptMask* keep = nullptr;
   if (fb->band_captured && !(keep = new (std::nothrow) KeptMask)) return false;
+  const OutsideCaptures outside;
   uint32_t* m = nullptr;
   if (cudaMalloc(&m, words * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();

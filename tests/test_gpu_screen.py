@@ -210,3 +210,34 @@ def test_words_memory_only_after_random_order(gpu):
             assert left[1] == left[0] and left[3] == left[2]
             assert (left[2] < left[1]) == (order == "shuffled")
         fb.close()
+
+
+def test_words_memory_while_another_stream_is_captured(gpu):
+    """A frame that takes the words' memory, on a stream of its own, leaves a capture in progress on another stream (in the
+    global mode, torch's default) as it is."""
+    import torch
+    n = 97 * 152 * 8 * 64 + 4321
+    pts = scenes.lidar(n, 49)
+    scenes.shuffle(pts, 2)
+    dev, v, side = _dev(pts), scenes.lidar_1km_view(400, 225), torch.cuda.Stream()
+    want = _frames(gpu, dev, v, 0, 1.0, (1, 100), tuning={"blocks_per_sm": 1})
+    x = torch.zeros(1000, device="cuda")
+    for frames_before in (0, 1):
+        fb = gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ)
+        gpu.pcr_set_tuning(fb, blocks_per_sm=1)
+        for _ in range(frames_before):
+            gpu.pcr_render_hq_splat(fb, dev, _view(v))
+        gpu.pcr_clear(fb)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            x += 1
+            gpu.pcr_render_hq_splat(fb, dev, _view(v), stream=side)
+            x += 1
+        graph.replay()
+        torch.cuda.synchronize()
+        keys, acc = gpu.pcr_framebuffer_keys(fb)
+        assert torch.equal(keys, want[0]) and torch.equal(acc, want[1])
+        del graph
+        fb.close()
+    assert float(x[0]) == 4.0
