@@ -350,8 +350,9 @@ typedef struct {
   int32_t slice_words;       /* batch kernel work item: 1 (default), 2 or 4 words of a view's chunk mask
                                 (32, 64 or 128 chunks of 1024 points); halved, down to one chunk, while a frame has
                                 too few items for the grid */
-  int32_t points_per_thread; /* points a thread classifies per step of the batch kernel: 1 (default) or 2; while no
-                                tuning has been set, pass 1 takes 2 */
+  int32_t points_per_thread; /* points a thread classifies per step of the batch kernel: 1 (default) or 2. A pass 1
+                                without merging takes 2 either way (faster at every size), and the screened pass 2
+                                of large clouds (pcr_batch_render) is not affected */
   int32_t blocks_per_sm;     /* 256-thread blocks per SM of the batch kernel, 1..32 (default 4; capped at the
                                 blocks that can be resident) */
   int32_t merge_width;       /* 0 (default): one atomic per fragment; 8, 16 or 32: fragments of aligned groups of

@@ -148,8 +148,7 @@ struct BatchTuning {
   int route = 0;              // 0: automatic (per-view passes for few views or large clouds), 1: batch kernel,
                               // 2: one single-view pass per view
   int slice_words = 1;        // mask words (32 chunks each) per work item: 1, 2 or 4
-  int points_per_thread = 1;  // points a thread classifies per step: 1 or 2
-  bool auto_points = true;    // not chosen by the caller: pass 1 takes 2 (see batch_points)
+  int points_per_thread = 1;  // points a thread classifies per step: 1 or 2 (see batch_points)
   int blocks_per_sm = 4;      // capped at the blocks that can be resident
   int merge_width = 0;        // 0: one atomic per fragment; 8, 16 or 32: same-pixel fragments of that many
                               // lanes merged first
@@ -309,11 +308,13 @@ __global__ void __launch_bounds__(kCertThreads, PCR_BATCH_MIN_BLOCKS) k_batch_pa
 // block: 0.49, 8: 0.46), 20M unchanged.
 constexpr int kMinItems = 4;
 
-// Points a thread takes per step. Unless the caller chose, pass 1 takes 2, whose key reads are in flight together: 16
-// views of mixed sizes on one GB300, 1 and 2 points: 1M points 327 and 321 us, 6M 769 and 747, 20M 1888 and 1818.
+// Points a thread takes per step: those of the tuning, but 2 for a pass 1 without merging, whose key reads are then in
+// flight together. 16 views of mixed sizes on one GB300, pass 1 with 1 and 2 points: basic frames of 300,000 points 251 and
+// 249 us, 1M 325 and 321, 6M 775 and 754, 20M 1891 and 1826; high-quality ones 3M 1122 and 1111, 20M 3722 and 3655. (Pass 2:
+// 1M 727 and 715; 3M 1122 and 1146, 20M 3722 and 4221 against the screened pass with one point in pass 1.)
 template <bool kHq>
 inline int batch_points(const BatchTuning& t) {
-  return t.auto_points ? (kHq ? 1 : 2) : t.points_per_thread;
+  return !kHq && t.merge_width == 0 ? 2 : t.points_per_thread;
 }
 
 // Launches the batch pass kernel of a tuning (template instance by merging and points per thread).
@@ -333,6 +334,8 @@ inline void batch_pass_launch(const BatchTuning& t, int sms, int resident, const
                                                         next_item, eps_num, eps_den, sc, mw)
   if (t.merge_width > 0) {
     if (batch_points<kHq>(t) == 2) PCR_BATCH_LAUNCH(true, 2); else PCR_BATCH_LAUNCH(true, 1);
+  } else if constexpr (!kHq) {
+    PCR_BATCH_LAUNCH(false, 2);
   } else {
     if (batch_points<kHq>(t) == 2) PCR_BATCH_LAUNCH(false, 2); else PCR_BATCH_LAUNCH(false, 1);
   }
@@ -348,10 +351,10 @@ inline int batch_pass_resident(const BatchTuning& t) {
     e = batch_points<kHq>(t) == 2
             ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, true, 2>, kCertThreads, 0)
             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, true, 1>, kCertThreads, 0);
+  else if (!kHq || batch_points<kHq>(t) == 2)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, false, 2>, kCertThreads, 0);
   else
-    e = batch_points<kHq>(t) == 2
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, false, 2>, kCertThreads, 0)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<kHq, false, 1>, kCertThreads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_pass<true, false, 1>, kCertThreads, 0);
   if (e != cudaSuccess || b < 1) {
     cudaGetLastError();
     b = 1;

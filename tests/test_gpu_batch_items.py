@@ -69,3 +69,30 @@ def test_captured_views_of_the_screened_pass(gpu):
             gpu.pcr_resolve(one, want, 0xFF010203, clear_after=True)
             assert torch.equal(o, want)
     batch.close()
+
+
+@pytest.mark.parametrize("n", [2_499_999, 2_500_000])
+def test_launches_follow_the_size_not_the_points_per_thread(gpu, n):
+    """From 2.5M points on, a high-quality frame's pass 2 is one launch per view, with the default tuning, with the same
+    tuning read and set again, and with two points per thread; the tuning read back is the one set."""
+    import torch
+    dev = torch.from_numpy(scenes.lidar(n, 63).view("int32")).cuda()
+    views = scenes.orbit_views(6, 3, resolutions=((200, 120), (333, 95)))
+    fbs = [gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ) for v in views]
+    outs = [torch.zeros(v.width * v.height, dtype=torch.int32, device="cuda") for v in views]
+    batch = gpu.pcr_batch_create(gpu.pcr_cloud_create(dev), fbs, outs, True, 1, 100, 0, True)
+    gpu.pcr_batch_set_views(batch, views)
+    default = gpu.pcr_batch_get_tuning(batch)
+    images = []
+    for tuning in (None, default, {"route": 1}, {"route": 1, "points_per_thread": 2}):
+        gpu.pcr_batch_set_tuning(batch, tuning)
+        assert gpu.pcr_batch_get_tuning(batch) == {**default, **(tuning or {})}
+        before = gpu.pcr_kernel_launch_count()
+        gpu.pcr_batch_render(batch)
+        # cull, tables, pass 1, pass 2, resolve
+        assert gpu.pcr_kernel_launch_count() - before == 4 + (len(views) if n >= 2_500_000 else 1), tuning
+        torch.cuda.synchronize()
+        images.append([o.clone() for o in outs])
+    for other in images[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(images[0], other))
+    batch.close()
