@@ -96,3 +96,26 @@ def test_launches_follow_the_size_not_the_points_per_thread(gpu, n):
     for other in images[1:]:
         assert all(torch.equal(a, b) for a, b in zip(images[0], other))
     batch.close()
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 5 * 1024, 31 * 1024 + 7, 32 * 1024, 33 * 1024 + 1, 700_001])
+@pytest.mark.parametrize("hq", [False, True])
+@pytest.mark.parametrize("tuning", [None, {"route": 1, "points_per_thread": 2}, {"route": 1, "merge_width": 32}])
+def test_items_of_other_tunings(gpu, n, hq, tuning):
+    import torch
+    dev = torch.from_numpy(scenes.lidar(n, 64).view("int32")).cuda()
+    views = scenes.orbit_views(6, 3, resolutions=((200, 120), (333, 95)))
+    flags = gpu.PCR_FB_HQ if hq else 0
+    fbs = [gpu.pcr_create_framebuffer(v.width, v.height, flags) for v in views]
+    outs = [torch.zeros(v.width * v.height, dtype=torch.int32, device="cuda") for v in views]
+    batch = gpu.pcr_batch_create(gpu.pcr_cloud_create(dev), fbs, outs, hq, 1, 100, 0, False)
+    gpu.pcr_batch_set_views(batch, views)
+    if tuning:
+        gpu.pcr_batch_set_tuning(batch, tuning)
+    gpu.pcr_batch_render(batch)
+    for v, fb in zip(views, fbs):
+        one = gpu.pcr_create_framebuffer(v.width, v.height, flags)
+        (gpu.pcr_render_hq_splat if hq else gpu.pcr_render_atomicmin)(one, dev, v)
+        for a, b in zip(gpu.pcr_framebuffer_keys(fb), gpu.pcr_framebuffer_keys(one)):
+            assert (a is None and b is None) or torch.equal(a, b)
+    batch.close()

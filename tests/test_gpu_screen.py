@@ -241,3 +241,87 @@ def test_words_memory_while_another_stream_is_captured(gpu):
         del graph
         fb.close()
     assert float(x[0]) == 4.0
+
+
+@pytest.mark.parametrize("tiles", [95, 96])
+@pytest.mark.parametrize("cloud", ["scan", "shuffled", "away"])
+def test_sampled_loops(gpu, cloud, tiles):
+    """Clouds on both sides of the sample's line, in tiles a warp of the device at hand, that every block finds in random
+    order (the second frame then takes pass 1's words), mostly outside the clip planes, or neither; the restated decision
+    says which loop ran."""
+    import torch
+    from tests.test_screen_restated import SAMPLE_TILES, sample_decisions
+    blocks, warps = torch.cuda.get_device_properties(0).multi_processor_count, 8
+    pts = scenes.lidar(tiles * blocks * warps * 64 + 17, 51)
+    if cloud == "shuffled":
+        scenes.shuffle(pts, 4)
+    v = scenes.lidar_1km_view(320, 180)
+    if cloud == "away":
+        v = scenes.View.lookat((500, 500, 60), (1500, 500, 40), (0, 0, 1), 60.0, 320, 180, 0.1, 100.0)
+    found = sample_decisions(pts, v, blocks, warps)
+    assert (found is None) == (tiles < SAMPLE_TILES)
+    if found is not None:
+        assert found[0].all() if cloud == "away" else not found[0].any()
+        assert cloud == "away" or (found[1].all() if cloud == "shuffled" else not found[1].any())
+    dev, one = _dev(pts), {"blocks_per_sm": 1}
+    want = _frames(gpu, dev, v, 0, 1.0, (1, 100), tuning=one)
+    fb = gpu.pcr_create_framebuffer(v.width, v.height, gpu.PCR_FB_HQ)
+    gpu.pcr_set_tuning(fb, **one)
+    for _ in range(3):
+        gpu.pcr_clear(fb)
+        gpu.pcr_render_hq_splat(fb, dev, _view(v))
+        torch.cuda.synchronize()
+        for a, b in zip(gpu.pcr_framebuffer_keys(fb), want):
+            assert torch.equal(a, b)
+    fb.close()
+
+
+RANGES = {1: [[0.0, 5000.0, 2e8]], 2: [[0.0, 4.0, 1e9], [4.0, 5000.0, 1e6]],
+          3: [[0.0, 2.0, 1e9], [2.0, 4.0, 1e11], [4.0, 5000.0, 1e3]],
+          5: [[0.0, 1.0, 1e8], [1.0, 3.0, 1e3], [3.1, 3.2, 1e9], [3.2, 3.5, 1e11], [3.5, 5000.0, 1e4]]}
+
+
+def _piecewise_keys(gpu, dev, v, ranges, before=None):
+    """Keys of one pass 1 by the exact and by the FP64 transform."""
+    res = []
+    for transform in (0, 1):
+        fb = gpu.pcr_create_framebuffer(v.width, v.height)
+        if before:
+            before(fb)
+        gpu.pcr_render_atomicmin(fb, dev, RawView(np.asarray(v.view_proj), v.near, v.far, v.width, v.height, 2, 1000.0,
+                                                  np.asarray(ranges), transform))
+        res.append(gpu.pcr_framebuffer_keys(fb)[0].clone())
+        fb.close()
+    assert int((res[0] != res[1]).sum()) == 0
+    return res[0]
+
+
+@pytest.mark.parametrize("n_ranges", sorted(RANGES))
+@pytest.mark.parametrize("spread", [0.0, 1e-7, 1e-4, 1.0])
+def test_piecewise_codes_next_to_the_stored_one(gpu, spread, n_ranges):
+    """As test_codes_next_to_the_stored_one, PIECEWISE: sheets inside a range, at a boundary and across all of them, on
+    empty keys and on keys that another mapping left."""
+    rng = np.random.default_rng(11)
+    n = 100_000
+    v = axis_view(64, 48)
+    for centre in (2.9, 3.2, 4.0):
+        w = centre * (1.0 + spread * (rng.random(n) - 0.5))
+        ndc = np.repeat(rng.uniform(-0.9, 0.9, (n // 50, 2)), 50, axis=0) + rng.uniform(0, 1e-3, (n, 2))
+        pts = pack(np.column_stack([ndc[:, 0] * w, ndc[:, 1] * w, -w]), rng.integers(0, 1 << 32, n, dtype=np.uint64))
+        for _ in range(2):
+            dev = _dev(pts)
+            keys = _piecewise_keys(gpu, dev, v, RANGES[n_ranges])
+            assert int((keys != -1).sum()) > 0
+            _piecewise_keys(gpu, dev, v, RANGES[n_ranges], lambda fb: gpu.pcr_render_atomicmin(fb, dev, v))
+            rng.shuffle(pts)
+
+
+@pytest.mark.parametrize("n_ranges", sorted(RANGES))
+def test_piecewise_special_coordinates(gpu, n_ranges):
+    pts = scenes.lidar(200_000, 52)
+    f = pts[:, :3].view(np.float32)
+    rng = np.random.default_rng(12)
+    for value in (np.nan, np.inf, -np.inf, 3e38, -3e38, 1e20, 1e-42, 0.0, -0.0):
+        f[rng.integers(0, len(pts), 800), rng.integers(0, 3, 800)] = value
+    scale = np.array([[250.0, 250.0, 1 / 250.0]])  # the same codes over 250 times the depth
+    _piecewise_keys(gpu, _dev(pts), scenes.lidar_1km_view(320, 180), np.asarray(RANGES[n_ranges]) * scale)
