@@ -172,17 +172,17 @@ pcr_status after_launch(const char* what, uint64_t launches = 1) {
   return e == cudaSuccess ? PCR_OK : cuda_fail(e, what);
 }
 
-// One word of pinned host memory per HQ framebuffer, in which pass 1 of a large frame leaves whether it found the cloud in
-// random order; a later frame reads it without waiting for anything. From one page for the process (null when its words
-// are all taken or it cannot be had).
-constexpr int kHints = 1024;
+// One 8-byte slot of pinned host memory per HQ framebuffer, whose first word pass 1 of a large frame sets when it finds the
+// cloud in random order; a later frame reads it without waiting for anything. From one page for the process (null when
+// its slots are all taken or it cannot be had).
+constexpr int kHints = 512;
 std::mutex g_hint_mu;
-uint32_t* g_hint_page = nullptr;
+uint64_t* g_hint_page = nullptr;
 bool g_hint_taken[kHints] = {};
 
 volatile uint32_t* take_hint() {
   std::lock_guard<std::mutex> lock(g_hint_mu);
-  if (!g_hint_page && cudaHostAlloc((void**)&g_hint_page, kHints * sizeof(uint32_t),
+  if (!g_hint_page && cudaHostAlloc((void**)&g_hint_page, kHints * sizeof(uint64_t),
                                     cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
     cudaGetLastError();
     g_hint_page = nullptr;
@@ -192,7 +192,7 @@ volatile uint32_t* take_hint() {
     if (!g_hint_taken[i]) {
       g_hint_taken[i] = true;
       g_hint_page[i] = 0u;
-      return g_hint_page + i;
+      return reinterpret_cast<uint32_t*>(g_hint_page + i);
     }
   return nullptr;
 }
@@ -200,7 +200,7 @@ volatile uint32_t* take_hint() {
 void give_hint(volatile uint32_t* hint) {
   if (!hint) return;
   std::lock_guard<std::mutex> lock(g_hint_mu);
-  g_hint_taken[hint - g_hint_page] = false;
+  g_hint_taken[reinterpret_cast<volatile uint64_t*>(hint) - g_hint_page] = false;
 }
 
 // A band mask request for pass 1: on, its eps, and where the launch's first tile sits in the mask (a pass 1
@@ -360,8 +360,9 @@ pcr_status render_hq(pcr_framebuffer* fb, const pcr_point* d_points, uint64_t n,
     // memory for pass 1's words only once a frame has found its cloud in random order: in scan order they are not written,
     // and the allocation takes 95 us (first frame of a framebuffer, 100M scanned points: 1034 us with it, 938 without)
     const bool words = fb->random_hint && *fb->random_hint && band_reserve(fb, n, s);
-    pcr::launch_raster_screen(pts, n, *P, S, fb->keys, words ? reinterpret_cast<uint2*>(fb->band_mask) : nullptr,
-                              const_cast<uint32_t*>(fb->random_hint), sms, per_sm, s);
+    pcr::launch_raster_screen(pts, n, *P, S, fb->keys,
+                              words ? pcr::kWords : fb->random_hint ? pcr::kOrder : pcr::kNothing,
+                              words ? (void*)fb->band_mask : (void*)fb->random_hint, sms, per_sm, s);
     pcr::HqScreenLaunch l;
     pcr::make_hq_screen(pts, n, *P, S, fb->keys, reinterpret_cast<unsigned long long*>(fb->accum), eps_num, eps_den,
                         words ? pcr::kBandWords : pcr::kAllTiles, words ? fb->band_mask : nullptr, sms, per_sm, &l);

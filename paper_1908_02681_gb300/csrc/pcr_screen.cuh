@@ -358,7 +358,7 @@ __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint
 //     each tile for lying outside as a whole before the pixel work. 400M city points on one GB300: 1.32 to 1.11 ms; done
 //     always, the test costs the 100M-point scan 2 % of pass 1 and piecewise depth 6 %.
 //   random: fewer than one in 64 of the sampled visible points share their pixel with the next point (clouds in no
-//     order): in HQ frames, pass 1 leaves pass 2 words that say which points it may accept (kBand). Pixels meet their
+//     order): in HQ frames, pass 1 leaves pass 2 words that say which points it may accept (kWords). Pixels meet their
 //     nearest points early then, and pass 2 reads 38 % of 37M shuffled points: the frame 0.44 to 0.38 ms on one GB300. In scan order
 //     the words leave 60 to 80 % of the points and cost more than they save (100M points 0.94 to 1.00 ms).
 // A block's decision depends on the cloud, the view and the launch shape alone: pass 2, of the same shape, comes to the
@@ -467,13 +467,16 @@ __device__ __forceinline__ void band_points(const uint4* __restrict__ pts, uint6
 // k_raster_cert, which computes every point's code, on one GB300: 400M city points at 4K 2.23 to 1.10 ms (the culled
 // points), 37M shuffled 0.227 to 0.18, 100M in scan order 0.539 to 0.48, and frames of 0.5 to 4 points per pixel equal
 // or a few per cent faster, so it runs at every size.
-// hint (HQ frames, or null): receives whether the sample found the cloud in random order.
-// kBand (HQ frames): also writes, per tile, a bit for each point that pass 2 may accept: clear where the point is culled or
-// certainly beyond the upper band edge of the key its pixel holds (a stored key only decreases, and the edge with it).
-template <int kMode, bool kBand>
+// kLeave (HQ frames): what else the pass leaves where `side` points. kOrder: one word, 1 where the sample finds the cloud in
+// random order (an instance of its own: in the plain one the argument cost 1M points 1.6 %). kWords: per tile, two words with
+// a bit for each point that pass 2 may accept, clear where the point is culled or certainly beyond the upper band edge of the
+// key its pixel holds (a stored key only decreases, and the edge with it).
+enum RasterLeave : int { kNothing = 0, kOrder = 1, kWords = 2 };
+
+template <int kMode, int kLeave>
 __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
     const uint4* __restrict__ pts, uint64_t n, const __grid_constant__ CertParams P, const __grid_constant__ Screen S,
-    unsigned long long* __restrict__ keys, uint2* __restrict__ band, uint32_t* __restrict__ hint) {
+    unsigned long long* __restrict__ keys, uint2* __restrict__ side) {
   extern __shared__ __align__(16) unsigned char smem[];
   long long* const sF = reinterpret_cast<long long*>(smem);
   const int tables = kMode >= kPiecewise2 ? P.n_pw : 1;
@@ -484,7 +487,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
   build_tables(P.col, tables, sF);
   wait_previous();
   const CloudSample sample = sample_cloud<kMode>(P, pts, n, T, lane);
-  if (kMode < kPiecewise2 && hint && T.g == 0u && lane == 0u) *hint = sample.random ? 1u : 0u;
+  if (kLeave == kOrder && sample.random && T.g == 0u && lane == 0u) side->x = 1u;
   uint32_t cn = 0, on = 0;
   auto tier2 = [&](uint32_t place) { raster_deferred(P, sF, point_at(pts, T, place), keys); };
   auto commit = [&](bool need, const uint4& p, uint32_t pixel, uint32_t place) {
@@ -496,7 +499,7 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
   auto candidate = [&](uint32_t i, bool valid) { commit(valid, q.p[i], q.pixel[i], q.place[i]); };
   auto record = [&](bool b0, bool b1, uint32_t place) {
     const unsigned m0 = __ballot_sync(0xFFFFFFFFu, b0), m1 = __ballot_sync(0xFFFFFFFFu, b1);
-    if (lane == 0) band[T.g + (uint64_t)(place >> 6) * T.G] = make_uint2(m0, m1);
+    if (lane == 0) side[T.g + (uint64_t)(place >> 6) * T.G] = make_uint2(m0, m1);
   };
   auto tile = [&](const uint4& p0, const uint4& p1, uint32_t place, bool words) {
         const ScreenTwo two = screen_two<kMode>(P, S, p0, p1, keys);
@@ -521,13 +524,13 @@ __global__ void __launch_bounds__(kScreenThreads, 1) k_raster_screen(
         if ((on | cn) >= 32u) drain_batches(q, on, cn, lane, tier2, candidate);
       };
   auto rest = [&](uint32_t place, bool v0, bool v1) {
-    if (kBand && sample.random) record(v0, v1, place);
+    if (kLeave == kWords && sample.random) record(v0, v1, place);
     push_open(v0, place, q.open, on, lane);
     push_open(v1, place + 32u, q.open, on, lane);
     drain_batches(q, on, cn, lane, tier2, candidate);
   };
   auto plain = [&](const uint4& p0, const uint4& p1, uint32_t place) { tile(p0, p1, place, false); };
-  if (kBand && sample.random)
+  if (kLeave == kWords && sample.random)
     screen_tiles<false>(
         pts, n, T, lane, [&](const uint4& p0, const uint4& p1, uint32_t place) { tile(p0, p1, place, true); }, rest);
   else if (sample.far_out)
@@ -716,30 +719,32 @@ inline ScreenLaunch screen_launch(uint64_t n, int sms, int per_sm, int tables, b
                       screen_smem(warps, tables, hq)};
 }
 
-template <int kMode, bool kBand = false>
+template <int kMode, int kLeave = kNothing>
 inline void raster_screen_launch(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                                 unsigned long long* keys, uint2* band, uint32_t* hint, int sms, int per_sm, cudaStream_t s) {
+                                 unsigned long long* keys, uint2* side, int sms, int per_sm, cudaStream_t s) {
   constexpr int most = kMode == kPiecewise ? kMaxRanges : kMode == kPiecewise2 ? 2 : 1;
   static std::atomic<uint64_t> opted{0};
-  opt_in_shared(k_raster_screen<kMode, kBand>, screen_smem(kScreenThreads / 32, most, false), opted);
+  opt_in_shared(k_raster_screen<kMode, kLeave>, screen_smem(kScreenThreads / 32, most, false), opted);
   const ScreenLaunch L = screen_launch(n, sms, per_sm, table_blocks(P), false);
-  launch_after(k_raster_screen<kMode, kBand>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, band, hint);
+  launch_after(k_raster_screen<kMode, kLeave>, L.grid, L.threads, L.smem, s, pts, n, P, S, keys, side);
 }
 
-// band (HQ frames of LINEAR or METRIC views, with the screen of pass 2's eps): receives the tiles' words for pass 2, or null.
-// hint: see k_raster_screen.
+// leave, side: see k_raster_screen (other than kNothing: LINEAR or METRIC views, with the screen of pass 2's eps).
 inline void launch_raster_screen(const uint4* pts, uint64_t n, const CertParams& P, const Screen& S,
-                                 unsigned long long* keys, uint2* band, uint32_t* hint, int sms, int per_sm,
+                                 unsigned long long* keys, RasterLeave leave, void* side, int sms, int per_sm,
                                  cudaStream_t s) {
+  uint2* const to = static_cast<uint2*>(side);
   switch (screen_mode(P)) {
     case kUnit256:
-      return band ? raster_screen_launch<kUnit256, true>(pts, n, P, S, keys, band, hint, sms, per_sm, s)
-                  : raster_screen_launch<kUnit256>(pts, n, P, S, keys, nullptr, hint, sms, per_sm, s);
+      return leave == kWords   ? raster_screen_launch<kUnit256, kWords>(pts, n, P, S, keys, to, sms, per_sm, s)
+             : leave == kOrder ? raster_screen_launch<kUnit256, kOrder>(pts, n, P, S, keys, to, sms, per_sm, s)
+                               : raster_screen_launch<kUnit256>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
     case kUnit1:
-      return band ? raster_screen_launch<kUnit1, true>(pts, n, P, S, keys, band, hint, sms, per_sm, s)
-                  : raster_screen_launch<kUnit1>(pts, n, P, S, keys, nullptr, hint, sms, per_sm, s);
-    case kPiecewise2: return raster_screen_launch<kPiecewise2>(pts, n, P, S, keys, nullptr, nullptr, sms, per_sm, s);
-    case kPiecewise: return raster_screen_launch<kPiecewise>(pts, n, P, S, keys, nullptr, nullptr, sms, per_sm, s);
+      return leave == kWords   ? raster_screen_launch<kUnit1, kWords>(pts, n, P, S, keys, to, sms, per_sm, s)
+             : leave == kOrder ? raster_screen_launch<kUnit1, kOrder>(pts, n, P, S, keys, to, sms, per_sm, s)
+                               : raster_screen_launch<kUnit1>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+    case kPiecewise2: return raster_screen_launch<kPiecewise2>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
+    case kPiecewise: return raster_screen_launch<kPiecewise>(pts, n, P, S, keys, nullptr, sms, per_sm, s);
   }
 }
 
@@ -806,7 +811,7 @@ inline void launch_raster_default(const uint4* pts, uint64_t n, const CertParams
                                   uint32_t* status, int sms, int per_sm, cudaStream_t s) {
   Screen S;
   if (make_screen(P, 0, 0, false, &S))
-    launch_raster_screen(pts, n, P, S, keys, nullptr, nullptr, sms, per_sm, s);
+    launch_raster_screen(pts, n, P, S, keys, kNothing, nullptr, sms, per_sm, s);
   else
     raster_launch<false, false>(pts, n, P, keys, nullptr, status, sms, per_sm, s);
 }
