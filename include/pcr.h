@@ -114,9 +114,11 @@ typedef struct {
                                skips the others. The records are exact: a stored key only decreases, so a point
                                whose code is already beyond the band of the key its pixel held can never be
                                accepted. pcr_render_hq_splat and pcr_render_frame_host do the same between
-                               their two passes. 0 (default): nothing is recorded. It pays off when points come
-                               in random order (pass 2 about 17 % faster, the HQ frame about 5 %), not in scan
-                               order, where pass 1's extra work outweighs it; the autotuner tries both. The first
+                               their two passes. 0 (default): nothing is recorded. Among passes with another
+                               option set it pays off when points come in random order, not in scan order; the
+                               passes of default tuning, which find out for themselves (pcr_render_hq_splat),
+                               are faster than it in both (100M scanned points 0.94 against 1.26 ms, 37M shuffled
+                               ones 0.38 against 0.51); the autotuner tries both. The first
                                recording of n points allocates n / 8 bytes of device memory (not during stream
                                capture, where nothing is recorded beyond the memory that is there; memory that a
                                captured frame uses is kept when a larger frame outgrows it); a clear drops the
@@ -128,9 +130,9 @@ typedef struct {
                                the host finds eps_num * (2^40 + Nq) + eps_den * 2^40 <= 2^64 (the same decision
                                as the band test of pcr_render_hq_splat then). The first such pass allocates
                                16 B per pixel (not during stream capture: there the stored-key test is used).
-                               0 (default): the band test on the stored key. Faster for points in random order
-                               without band records (pass 2 about 1 %), slower in scan order (about 3 %); the
-                               autotuner tries both. */
+                               0 (default): the band test on the stored key, on a float depth first: faster
+                               in scan and random order (100M scanned points 0.94 against 1.22 ms, 37M shuffled
+                               ones 0.38 against 0.51); the autotuner tries both. */
 } pcr_tuning;
 
 /* Framebuffer flags. */
@@ -152,7 +154,8 @@ pcr_status pcr_set_tuning(pcr_framebuffer* fb, const pcr_tuning* tuning);
 pcr_status pcr_get_tuning(const pcr_framebuffer* fb, pcr_tuning* tuning);
 
 /* Autotuner: renders one frame of (d_points, n, view) on fb for every candidate tuning (same-pixel merging
- * on and off, both stagings, 2 / 4 / 6 / 8 blocks per SM, and for HQ framebuffers band records with eps 1/100
+ * on and off, both stagings, 2 / 4 / 6 / 8 blocks per SM (4, 6 and 8 are one launch shape for the passes of default
+ * tuning), and for HQ framebuffers band records with eps 1/100
  * and pass 2's per-pixel bounds, each on and off), times the point passes with CUDA events on `stream` (pass 1,
  * plus pass 2 with eps 1/100 for HQ framebuffers; best of two runs), and keeps the fastest in fb. Writes it
  * to *best when best is not NULL. Clears fb before every run and at the end; synchronises `stream`.
@@ -394,7 +397,8 @@ pcr_status pcr_batch_destroy(pcr_batch* batch);
 #define PCR_NOALLOC_MAX_POINTS 134217728ull /* 2^27 points (131072 chunks of 1024) */
 
 /* One batched frame of count views of n points: the same images as pcr_cloud_create + pcr_batch_create +
- * pcr_batch_set_views + pcr_batch_render (always with the batched persistent launch), but the frame's
+ * pcr_batch_set_views + pcr_batch_render (with the persistent launch whatever the number of views and points; a
+ * high-quality frame's pass 2 is one launch per view from 2.5 * 10^6 points on, as there), but the frame's
  * workspace (chunk bounds, visibility masks, per-view constants, counters) is a fixed device array inside libpcr, so
  * the call allocates nothing: no cudaMalloc, cudaFree or other allocating routine. It is meant for callers
  * that must not allocate while they render: a render loop in which a cudaMalloc or cudaFree would

@@ -79,9 +79,9 @@ __host__ __device__ __forceinline__ bool depth_entry(const DepthColumn& c, int e
 
 // Per-view constants of the certified evaluation. Passed by value as a __grid_constant__ kernel parameter (about
 // 1.9 KB), so concurrent launches with different views share nothing. The depth tables (12 KB a view or PIECEWISE
-// range) are not in it: every block builds them from the columns below (build_tables). They used to be built on the
-// host (14 us a view), copied to the device and read by each block: a frame with a new camera over 40,000 points took
-// 37 us that way and takes 26 us now, 1M points at 640x480 38 us and now 30 us.
+// range) are not in it: every block builds them from the columns below (build_tables). Built on the host they took 14 us
+// a view, a copy to the device and a read by each block: with nothing else different, a frame with a new camera over
+// 40,000 points took 37 us that way against 26, 1M points at 640x480 38 against 30.
 struct CertParams {
   // hot scalars first: the per-point loops read them as instruction operands; the columns come last
   float H[3][4], L[3][4];             // float splits of the rows clip x, clip y, w (H: nearest float, L: rest)

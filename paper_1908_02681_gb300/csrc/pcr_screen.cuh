@@ -352,15 +352,17 @@ __device__ __forceinline__ void screen_tiles(const uint4* __restrict__ pts, uint
   if (rem != 0u && n_full % G == g) rest(end, lane < rem, lane + 32u < rem);
 }
 
-// A pass over at least this many tiles a warp samples the cloud first, a tile a warp spread over all of it (1.5 us, 1 % of
-// a frame of 25M points, hence the line), and its blocks take the loop that suits it:
+// A pass over at least this many tiles a warp (2.99e7 points on 152 SMs with default tuning) samples the cloud first, a tile a
+// warp spread over all of it (1.5 us: 0.6 % of a high-quality frame of 28M scanned points, 1.1 % of 15M; shuffled clouds
+// below the line go without the words, which would take their frame at 22M points from 291 to 251 us and at 10M from 151 to
+// 139), and its blocks take the loop that suits it:
 //   far_out: a quarter of the sampled points lie outside the clip planes (scans much larger than the view): pass 1 tests
 //     each tile for lying outside as a whole before the pixel work. 400M city points on one GB300: 1.32 to 1.11 ms; done
 //     always, the test costs the 100M-point scan 2 % of pass 1 and piecewise depth 6 %.
 //   random: fewer than one in 64 of the sampled visible points share their pixel with the next point (clouds in no
-//     order): in HQ frames, pass 1 leaves pass 2 words that say which points it may accept (kWords). Pixels meet their
-//     nearest points early then, and pass 2 reads 38 % of 37M shuffled points: the frame 0.44 to 0.38 ms on one GB300. In scan order
-//     the words leave 60 to 80 % of the points and cost more than they save (100M points 0.94 to 1.00 ms).
+//     order): in HQ frames, from the one after that on, pass 1 leaves pass 2 words that say which points it may accept
+//     (kWords). Pixels meet their nearest points early then, and pass 2 reads 38 % of 37M shuffled points: the frame 0.46 to
+//     0.38 ms on one GB300. In scan order the words leave 60 to 80 % of the points and cost more than they save (100M points 0.94 to 1.00 ms).
 // A block's decision depends on the cloud, the view and the launch shape alone: pass 2, of the same shape, comes to the
 // same one for the same tiles.
 constexpr uint32_t kSampleTiles = 96;
